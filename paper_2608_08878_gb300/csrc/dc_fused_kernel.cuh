@@ -43,6 +43,15 @@
 // the V pass re-reads them, with the positions and |v| (L2-resident), in loads
 // issued two tiles ahead of use.
 //
+// The producer's copies and the MMAs are issued by the lane that elect.sync
+// picks, not by "lane 0": the compiler then knows that one thread runs and
+// keeps descriptors and coordinates in uniform registers, which these
+// instructions take. With lane 0 every operand was moved there one by one,
+// 694 + 1074 cycles of a tile's QK and PV issue (231 + 416 now, clock64 stamps
+// on 411-token rows), 640 + 564 of its two TMA issues (309 + 290): 8192-token
+// rows 1386 -> 1335 us a step (2048 rows), 411-token rows 774 -> 723 (16384
+// rows), one layer of 8 rows of 2049 tokens 28.9 -> 26.1.
+//
 // Barrier phases: a parity wait is only sound when the waiting thread cannot
 // be two phases ahead of the barrier. Every barrier here has one waiter that
 // waits its phases in order (the producer, the MMA issuer, one warpgroup), or,
@@ -478,9 +487,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     int g = 0, issued = 0;
     bool last = false;  // a half row was taken: nothing more
     for (int gr = 0;; ++gr) {
-      if (*abort) break;
+      // (the warp leaves the loop together, also when the kernel winds down)
+      if (__any_sync(0xffffffffu, *abort != 0)) break;
       const int qb = gr & 1;
-      if (!mbar_wait(&bar[B_QEMPTY + qb], ((gr >> 1) & 1) ^ 1, abort, p.dbg, 1u, (unsigned)gr)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(&bar[B_QEMPTY + qb], ((gr >> 1) & 1) ^ 1, abort, p.dbg, 1u, (unsigned)gr)))
+        break;
       // the next item, taken once this CTA's query buffer is free
       int4 iv = make_int4(-1, 0, 0, 0);
       if (lane == 0) {
@@ -565,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       fence_proxy_async();
       __syncwarp();
-      if (lane == 0) {
+      if (elect_one()) {
         mbar_arrive(&bar[B_QFULL + qb]);
         // PAIR: the two rows' tiles alternate (x even: the first row)
         const int nx = (PAIR ? 2 : 1) * (it.t1 - it.t0);
@@ -614,17 +625,19 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      g = __shfl_sync(0xffffffffu, g, 0);
-      issued = __shfl_sync(0xffffffffu, issued, 0);
     }
-    // every issued load must land before the CTA may exit
-    if (lane == 0) {
+    // every issued load must land before the CTA may exit (the elected lane is
+    // always the same: it alone counts the tiles)
+    if (elect_one()) {
       for (int t = issued - kStages < 0 ? 0 : issued - kStages; t < issued; ++t)
         mbar_wait_drain(&bar[B_FULL + t % kStages], (t / kStages) & 1);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
+      const uint32_t stage_lo = sdesc_lo(smem_u32(smem + OFF_STAGE), 16);
+      const uint32_t vstage_lo = sdesc_lo(smem_u32(smem + OFF_STAGE), 16384);
+      const uint32_t q_lo = sdesc_lo(smem_u32(smem + OFF_Q), 16), p_lo = sdesc_lo(smem_u32(smem + OFF_P), 4096);
       const uint32_t id_qk = idesc_bf16(128, NQ, 0, 0);
       const uint32_t id_pv = idesc_bf16(128, 16, 1, 1);
       int g = 0, gs = 0, gv = 0;
@@ -636,18 +649,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_after();
         const int nx = (PAIR ? 2 : 1) * (it.t1 - it.t0);  // PAIR: the rows' tiles alternate
         for (int x = 0; x < nx; ++x, ++g, ++gs) {
-          const uint32_t qaddr = smem_u32(smem + OFF_Q + (PAIR ? 2 * qb + (x & 1) : qb) * L::QBYTES);
+          const uint32_t qlo = q_lo + (uint32_t)(PAIR ? 2 * qb + (x & 1) : qb) * (L::QBYTES >> 4);
           const int s = g % kStages, b = gs & 1;
           if (!mbar_wait(&bar[B_FULL + s], (g / kStages) & 1, abort, p.dbg, 4u, (unsigned)g)) break;
           if (!mbar_wait(&bar[B_SEMPTY + b], ((gs >> 1) & 1) ^ 1, abort, p.dbg, 5u, (unsigned)gs)) break;
           tc_fence_after();
-          const uint32_t kaddr = smem_u32(smem + OFF_STAGE + s * kStageBytes);
+          const uint32_t klo = stage_lo + (uint32_t)s * (kStageBytes >> 4);
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
             const uint32_t off = (uint32_t)(ks >> 2) * 16384u + (uint32_t)(ks & 3) * 32u;
             const uint32_t qoff = (uint32_t)(ks >> 2) * (uint32_t)(NQ * 128) + (uint32_t)(ks & 3) * 32u;
-            mma_bf16(tmem + kColS + b * NQ, sdesc_sw128(kaddr + off, 16, 1024), sdesc_sw128(qaddr + qoff, 16, 1024),
-                     id_qk, ks > 0);
+            mma_bf16_lo(tmem + kColS + b * NQ, klo + (off >> 4), sdesc_hi(1024, 2), qlo + (qoff >> 4), sdesc_hi(1024, 2),
+                        id_qk, ks > 0);
           }
           mma_commit(&bar[B_SFULL + b]);
           mma_commit(&bar[B_EMPTY + s]);
@@ -667,13 +680,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!mbar_wait(&bar[B_PFULL + pb], (gv >> 1) & 1, abort, p.dbg, 14u, (unsigned)gv)) break;
           if (x == 0 && !mbar_wait(&bar[B_OEMPTY], (gr & 1) ^ 1, abort, p.dbg, 15u, (unsigned)gr)) break;
           tc_fence_after();
-          const uint32_t vaddr = smem_u32(smem + OFF_STAGE + s * kStageBytes);
-          const uint32_t paddr = smem_u32(smem + OFF_P + pb * 4096);
+          const uint32_t vlo = vstage_lo + (uint32_t)s * (kStageBytes >> 4);
+          const uint32_t plo = p_lo + (uint32_t)pb * (4096 >> 4);
           // O^T[d x 16] += V^T[d x 128] P^T: V^T is MN-major (dims contiguous)
 #pragma unroll
           for (int ks = 0; ks < kTok / 16; ++ks)
-            mma_bf16(tmem + ocol, sdesc_sw128(vaddr + ks * 2048u, 16384, 1024),
-                     sdesc_sw32(paddr + ks * 512u, 4096, 256), id_pv, (!first || ks > 0) ? 1u : 0u);
+            mma_bf16_lo(tmem + ocol, vlo + ks * (2048u >> 4), sdesc_hi(1024, 2), plo + ks * (512u >> 4), sdesc_hi(256, 6),
+                        id_pv, (!first || ks > 0) ? 1u : 0u);
           mma_commit(&bar[B_PEMPTY + pb]);
           mma_commit(&bar[B_EMPTY + s]);
           if (x == nx - 1) mma_commit(&bar[B_OFULL]);
@@ -686,9 +699,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == 10) {
     // ------------------------------------------------------------ policy-layer MMA issuer
-    if (!FULL && !HEUR && !GLOB && lane == 0) {
+    if (!FULL && !HEUR && !GLOB && elect_one()) {
       const uint32_t id_m = idesc_bf16(128, 128, 0, 0);
-      const uint32_t waddr = smem_u32(smem + OFF_W);
+      const uint32_t wlo = sdesc_lo(smem_u32(smem + OFF_W), 16), a_lo = sdesc_lo(smem_u32(smem + OFF_A), 16);
       int gv = 0;
       for (int gr = 0;; ++gr) {
         const Item it = read_item(items, gr, abort, p.dbg, 24u);
@@ -699,12 +712,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (!mbar_wait(&bar[B_AFULL + pb], (gv >> 1) & 1, abort, p.dbg, 16u, (unsigned)gv)) break;
           if (!mbar_wait(&bar[B_MEMPTY + pb], ((gv >> 1) & 1) ^ 1, abort, p.dbg, 17u, (unsigned)gv)) break;
           tc_fence_after();
-          const uint32_t aaddr = smem_u32(smem + OFF_A + pb * 8192);
+          const uint32_t alo = a_lo + (uint32_t)pb * (8192 >> 4);
           // Z[128 x 128] = A[128 x 32] W^T
 #pragma unroll
           for (int ks = 0; ks < 2; ++ks)
-            mma_bf16(tmem + kColM + pb * 128, sdesc_sw64(aaddr + ks * 32u, 16, 512),
-                     sdesc_sw64(waddr + ks * 32u, 16, 512), id_m, ks > 0);
+            mma_bf16_lo(tmem + kColM + pb * 128, alo + ks * (32u >> 4), sdesc_hi(512, 4), wlo + ks * (32u >> 4),
+                        sdesc_hi(512, 4), id_m, ks > 0);
           mma_commit(&bar[B_MFULL + pb]);
           mma_commit(&bar[B_AEMPTY + pb]);
         }
