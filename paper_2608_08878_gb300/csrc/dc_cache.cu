@@ -611,6 +611,7 @@ dc::FusedStep fused_args(dc_cache* h, const dc::Step& st, const void* q, float* 
   fs.xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
   fs.work = h->work;
   fs.half_rows = (h->xflag && !h->per_row) ? dc::fused_half_rows(h->dev, st.n, fs, h->num_sms) : 0;
+  fs.batch_rows = dc::fused_batch_rows(h->dev, st.n, h->num_sms);
   // launch epoch: the queue counter is work[epoch & 1]; exchange flags hold
   // epoch * 4 + phase (1..3), so a flag left by an earlier launch never matches
   fs.epoch = ++h->epoch;
@@ -638,6 +639,7 @@ dc_status graph_step(dc_cache* h, const void* q, const void* k_new, const void* 
   fs.xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
   fs.work = h->work;
   fs.half_rows = h->xflag ? dc::fused_half_rows(h->dev, h->gstep.n, fs, h->num_sms) : 0;
+  fs.batch_rows = dc::fused_batch_rows(h->dev, h->gstep.n, h->num_sms);
   fs.epoch = h->gepoch;
   cudaError_t e;
   {
@@ -891,7 +893,7 @@ dc_status dc_step_host_async(dc_cache* h, const void* q, const void* k_new, cons
 dc_status dc_engine(dc_cache* h, int n, int* engine) {
   if (!valid(h) || !engine) return DC_ERR_INVALID_ARG;
   const int nn = n > 0 ? n : h->n + 1;
-  *engine = !use_fused(h, nn) ? 1 : dc::fused_pairs(h->dev, nn, h->num_sms) ? 3 : 2;
+  *engine = !use_fused(h, nn) ? 1 : dc::fused_batch_rows(h->dev, nn, h->num_sms) ? 3 : 2;
   return DC_OK;
 }
 

@@ -40,6 +40,7 @@ struct FusedStep {
   int* xsel;         // [half_rows][2][4]
   unsigned* xflag;   // [half_rows][2]
   int xslots;        // exchange slots allocated (bounds of the four above)
+  int batch_rows;    // rows per work item when the step runs on batches of rows (batch_kernel), else 0
 };
 
 // Exchange buffer sizes (floats / ints) for a grid of `grid` CTAs.
@@ -79,16 +80,19 @@ cudaError_t make_fused_maps(const Dev& p, FusedMaps* maps, const char** why);
 // FusedPolicy fields and the host copy of the weight tile (128 * 32 bf16).
 void prepare_policy(const float* blob, int H, int layernorm, FusedPolicy* fp, std::vector<__nv_bfloat16>* wtile);
 
-// Whether a step over n tokens runs on row pairs (each warpgroup of a CTA on
-// its own row): short rows (at most kPairTiles tiles), more rows than SMs, an
-// even row count, the plain step (policy scorer, equal lengths, per-row
-// selection).
-bool fused_pairs(const Dev& p, int n, int num_sms);
+// Rows per work item when a step over n tokens runs on batches of rows (each
+// warpgroup of a CTA on rows of its own, dc_batch_kernel.cuh), 0 when it does
+// not: short rows, more rows than SMs, an even row count, the plain step
+// (policy scorer, equal lengths, per-row selection).
+int fused_batch_rows(const Dev& p, int n, int num_sms);
+// Tiles of a row that fit the batch schedule, and the rows per item there.
+int batch_row_tiles(int G);
+int batch_rows_per_item(const Dev& p, int n, int num_sms);
 
 // How many rows a step over n tokens splits into halves (see FusedStep): every
 // row when rows are at most half the SMs and at least 12 tiles long, else the
 // remainder of R over the grid when it is at most half the grid, else 0 (and 0
-// on row pairs).
+// on batches of rows).
 int fused_half_rows(const Dev& p, int n, const FusedStep& fs, int num_sms);
 
 cudaError_t launch_fused_step(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
@@ -101,12 +105,12 @@ cudaError_t launch_fused_heur_perrow(const FusedMaps& maps, const Dev& p, const 
                                      const FusedPolicy& fp, int num_sms, cudaStream_t s);
 cudaError_t launch_fused_glob(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                               const FusedPolicy& fp, int num_sms, cudaStream_t s);
-// Row pairs (dc_fused_pair.cu).
-cudaError_t launch_fused_pair(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
+// Batches of rows (dc_batch.cu), FusedStep::batch_rows > 0.
+cudaError_t launch_fused_batch(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                               const FusedPolicy& fp, int num_sms, cudaStream_t s);
 // Device-counted steps (dc_fused_graph.cu): st and fs.epoch are base values
-// that the kernel advances by Dev::gcount[0]; whole rows, halves or row pairs
-// (as the plain step would take them), policy scorer, one eviction per step.
+// that the kernel advances by Dev::gcount[0]; whole rows, halves or batches of
+// rows (as the plain step would take them), policy scorer, one eviction per step.
 cudaError_t launch_fused_graph(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                                const FusedPolicy& fp, int num_sms, cudaStream_t s);
 

@@ -13,7 +13,7 @@
 // One CTA per SM (or per row, or two per row: rows of 12 tiles or more are
 // split in halves when there are at most half as many rows as SMs); the CTAs
 // take rows, half rows (also for a partly filled last wave) or, on short rows,
-// row pairs (PAIR) from a shared queue as they become free. A row's ragged
+// batches of rows (dc_batch_kernel.cuh) as they become free. A row's ragged
 // last tile is loaded in boxes of 16 tokens.
 // Warp roles (352 threads):
 //   warp 0     producer: takes the next row, writes its query tile (current,
@@ -110,26 +110,18 @@ constexpr int max_tok() {
   return G == 8 ? 8192 : kFusedMaxTok;
 }
 
-// Row pairs (PAIR): an item is two rows of at most kPairTiles tiles, one per
-// warpgroup; their K and V tiles alternate in the stage ring.
-constexpr int kPairTiles = 21;
-constexpr int kPairTok = kPairTiles * kTok;
-constexpr int kColOB = 48;                                 // the second row's O (PAIR)
-constexpr int kPairStashA = 64;                            // the first row's logit stash (PAIR)
-
-// Shared memory layout; PAIR keeps four query tiles (two per item, double
-// buffered) and a smaller logit/score array per row.
-template <bool PAIR, int G>
+// Shared memory layout.
+template <int G>
 struct Smem {
   static constexpr int QBYTES = q_rows<G>() * 256;         // one query tile: two 64-dim blocks
   static constexpr int STAGE = 0;
-  static constexpr int Q = STAGE + kStages * kStageBytes;   // (2 or 4) query tiles
-  static constexpr int P = Q + (PAIR ? 4 : 2) * QBYTES;     // 2 x 4 KB (one per warpgroup)
+  static constexpr int Q = STAGE + kStages * kStageBytes;   // 2 query tiles
+  static constexpr int P = Q + 2 * QBYTES;     // 2 x 4 KB (one per warpgroup)
   static constexpr int A = P + 2 * 4096;                    // 2 x 8 KB (one per warpgroup)
   static constexpr int W = A + 2 * 8192;                    // 8 KB
   static constexpr int AUX = W + 8192;                      // kStages x 2560 B
   static constexpr int SC = AUX + kStages * kAuxBytes;      // head G-1 logits, then scores
-  static constexpr int MISC = SC + (PAIR ? 2 * kPairTok : max_tok<G>()) * 4;
+  static constexpr int MISC = SC + max_tok<G>() * 4;
   static constexpr int BYTES = MISC + 4096 + 1024;          // misc area + alignment slack
   static_assert(BYTES <= 232448, "more shared memory than a CTA may have");
 };
@@ -298,10 +290,9 @@ struct Item {
 
 constexpr int kItemRing = 8;  // items published ahead of the slowest role (at most ~3)
 
-template <bool PERROW, bool PAIR>
+template <bool PERROW>
 __device__ __forceinline__ Item take_item(const FusedStep& fs, const Dev& p, int nT) {
   const unsigned w = atomicAdd(fs.work + (fs.epoch & 1u), 1u);
-  if constexpr (PAIR) return w < (unsigned)(p.R / 2) ? Item{(int)(2 * w), 0, nT, -1} : Item{-1, 0, 0, 0};
   const unsigned whole = (unsigned)(p.R - fs.half_rows);
   if (w < whole) {
     if (!PERROW) return Item{(int)w, 0, nT, -1};
@@ -356,21 +347,15 @@ __device__ __forceinline__ Item read_item(volatile int* ring, int gr, volatile i
 // GRAPH: device-counted steps: the step arguments are the host's base values
 // plus the number of steps taken since (Dev::gcount[0], advanced by the last
 // CTA to finish), so that a captured launch replays as the following steps.
-// PAIR: items are row pairs (rows 2w and 2w + 1) of at most kPairTiles tiles,
-// warpgroup w doing the whole of row 2w + w (its K and V tiles alternate with
-// the other row's in the ring), so that one row's merge, output and select
-// overlap the other's; policy scorer, whole rows, equal lengths only.
 // PERROW: rows of different lengths and budgets (Dev::rowlen, Dev::rowbudget;
 // FusedStep::B > 0 overrides every row's budget); the kernel writes each
 // row's new length after its selection. No half rows.
-template <int D, int G, bool LONG, bool FULL, bool HEUR, bool GLOB, bool PERROW, bool PAIR, bool GRAPH>
+template <int D, int G, bool LONG, bool FULL, bool HEUR, bool GLOB, bool PERROW, bool GRAPH>
 __global__ void __launch_bounds__(kThreads, 1)
     fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                  const __grid_constant__ CUtensorMap tmK16, const __grid_constant__ CUtensorMap tmV16, Dev p,
                  Step st, FusedStep fs, FusedPolicy fp) {
   constexpr int GS = G - 1;  // heads whose logits wait in TMEM between the passes
-  static_assert(!PAIR || (!LONG && !FULL && !HEUR && !GLOB && !PERROW), "row pairs: the plain step only");
-  static_assert(!PAIR || G <= 4, "row pairs: up to four query heads per KV head");
   constexpr int NQ = q_rows<G>();   // query-tile rows, S-tile columns
   constexpr int kColO = col_o<G>();
   // G = 8: the per-row statistics of the window's queries (the K pass) sit in
@@ -390,7 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     st.slot_prev = (st.slot_prev + t) % p.w;
     fs.epoch += (unsigned)t;
   }
-  using L = Smem<PAIR, G>;
+  using L = Smem<G>;
   constexpr int OFF_STAGE = L::STAGE, OFF_Q = L::Q, OFF_P = L::P, OFF_A = L::A, OFF_W = L::W, OFF_AUX = L::AUX,
                 OFF_SC = L::SC, OFF_MISC = L::MISC;
   extern __shared__ uint8_t smem_raw[];
@@ -399,10 +384,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   static_assert(8 * B_COUNT <= 384, "barriers overlap the misc fields");
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_MISC + 384);
   volatile int* abort = reinterpret_cast<volatile int*>(smem + OFF_MISC + 388);
-  // [8][G][3]; with G = 8 in the area the row pairs' scratch takes otherwise
+  // [8][G][3]; with G = 8 further back
   float* red = reinterpret_cast<float*>(smem + OFF_MISC + (G == 8 ? 2560 : 512));
   float* s_wq = reinterpret_cast<float*>(smem + OFF_MISC + 3328);          // G = 8: [6][8], then [3][8]
-  static_assert(G != 8 || (!PAIR && 2560 + 8 * G * 3 * 4 <= 3328 && 3328 + 9 * 8 * 4 <= MISC_BYTES),
+  static_assert(G != 8 || (2560 + 8 * G * 3 * 4 <= 3328 && 3328 + 9 * 8 * 4 <= MISC_BYTES),
                 "misc area layout");
   int* s_hist = reinterpret_cast<int*>(smem + OFF_MISC + 1024);           // [256]
   int* s_sh = reinterpret_cast<int*>(smem + OFF_MISC + 2048);             // [4]
@@ -411,13 +396,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   int* s_best_slot = reinterpret_cast<int*>(smem + OFF_MISC + 2176);      // [8]
   float* sc = reinterpret_cast<float*>(smem + OFF_SC);
   volatile int* items = reinterpret_cast<volatile int*>(smem + OFF_MISC + 2304);  // [8][4] + seq [8]
-  // PAIR: the second warpgroup's select scratch
-  int* s_hist2 = reinterpret_cast<int*>(smem + OFF_MISC + 2560);          // [256]
-  int* s_sh2 = reinterpret_cast<int*>(smem + OFF_MISC + 3584);            // [4]
-  int* s_wsum2 = reinterpret_cast<int*>(smem + OFF_MISC + 3600);          // [4]
-  unsigned long long* s_best2 = reinterpret_cast<unsigned long long*>(smem + OFF_MISC + 3616);  // [4]
-  int* s_best_slot2 = reinterpret_cast<int*>(smem + OFF_MISC + 3648);     // [4]
-
   const int warp = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
   const int n_step = st.n, nT = (n_step + kTok - 1) / kTok;
   constexpr uint32_t kTileBytes = (uint32_t)D * kTok * 2;
@@ -440,7 +418,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&bar[B_AEMPTY + b], 1);
     }
     mbar_init(&bar[B_OFULL], 1);
-    mbar_init(&bar[B_OEMPTY], PAIR ? 8 : 4);
+    mbar_init(&bar[B_OEMPTY], 4);
     mbar_init(&bar[B_DRAIN], 1);
     mbar_init(&bar[B_DRAIN2], 1);
     *abort = 0;
@@ -495,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the next item, taken once this CTA's query buffer is free
       int4 iv = make_int4(-1, 0, 0, 0);
       if (lane == 0) {
-        const Item t = last ? Item{-1, 0, 0, 0} : take_item<PERROW, PAIR>(fs, p, nT);
+        const Item t = last ? Item{-1, 0, 0, 0} : take_item<PERROW>(fs, p, nT);
         publish_item(items, gr, t);
         iv = make_int4(t.row, t.t0, t.t1, t.half);
       }
@@ -507,46 +485,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (it.row < 0) break;
       last = it.half >= 0;
       const int r = it.row;
-      // query tile (PAIR: one per row): rows [0,G) current, [G,2G) previous
-      // step, [2G,3G) departing
-      if constexpr (PAIR) {
-        // row pairs: a row's loads issued together (every element is read
-        // before any is written, as the current query takes over the departing
-        // query's ring slot), one global round trip per row
-        constexpr int QCH = G * (D / 8);                 // 16-byte chunks of a row's G query heads
-        constexpr int QIT = (QCH + kWarp - 1) / kWarp;   // per lane
-        for (int qi = 0; qi < 2; ++qi) {
-          const int rq = r + qi;
-          uint8_t* qt = smem + OFF_Q + (2 * qb + qi) * L::QBYTES;
-          const int qo = ((rq / p.kvh) * p.qh + (rq % p.kvh) * G) * D;
-          const __nv_bfloat16* prev = p.ring_q + ((size_t)rq * p.w + st.slot_prev) * G * D;
-          const __nv_bfloat16* dep = p.ring_q + ((size_t)rq * p.w + st.slot) * G * D;
-          __nv_bfloat16* ring_slot = p.ring_q + ((size_t)rq * p.w + st.slot) * G * D;
-          const bool q_ok = DC_INB(p, qo + G * D - 1, (long long)(p.R / p.kvh) * p.qh * D, 101) &&
-                            DC_INB(p, ((long long)rq * p.w + st.slot) * G * D + G * D - 1, (long long)p.R * p.w * G * D, 102) &&
-                            DC_INB(p, ((long long)rq * p.w + st.slot_prev) * G * D, (long long)p.R * p.w * G * D, 103);
-          uint4 qcur[QIT], qprev[QIT], qdep[QIT];
-#pragma unroll
-          for (int u = 0; u < QIT; ++u) {
-            const int e = lane + u * kWarp;
-            const int h = e / (D / 8), kc = e % (D / 8);
-            const bool ld = q_ok && e < QCH;
-            qcur[u] = ld ? reinterpret_cast<const uint4*>(fs.q + qo + h * D)[kc] : make_uint4(0, 0, 0, 0);
-            qprev[u] = ld && st.has_prev ? reinterpret_cast<const uint4*>(prev + h * D)[kc] : make_uint4(0, 0, 0, 0);
-            qdep[u] = ld && st.has_dep ? reinterpret_cast<const uint4*>(dep + h * D)[kc] : make_uint4(0, 0, 0, 0);
-          }
-#pragma unroll
-          for (int u = 0; u < QIT; ++u) {
-            const int e = lane + u * kWarp;
-            if (!q_ok || e >= QCH) continue;
-            const int h = e / (D / 8), kc = e % (D / 8);
-            *reinterpret_cast<uint4*>(qt + (kc >> 3) * (NQ * 128) + sw128(h, kc & 7)) = qcur[u];
-            *reinterpret_cast<uint4*>(qt + (kc >> 3) * (NQ * 128) + sw128(G + h, kc & 7)) = qprev[u];
-            *reinterpret_cast<uint4*>(qt + (kc >> 3) * (NQ * 128) + sw128(2 * G + h, kc & 7)) = qdep[u];
-            if (!FULL && it.half < 0) reinterpret_cast<uint4*>(ring_slot + h * D)[kc] = qcur[u];  // halves: see the epilogue
-          }
-        }
-      } else {
+      // query tile: rows [0,G) current, [G,2G) previous step, [2G,3G) departing
+      {
         // whole rows: one chunk per lane at a time (on whole rows this measured
         // faster than issuing the row's loads together: 6.04 against 6.25 ms
         // per step at 64 x 16384 x 25%)
@@ -578,12 +518,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (elect_one()) {
         mbar_arrive(&bar[B_QFULL + qb]);
-        // PAIR: the two rows' tiles alternate (x even: the first row)
-        const int nx = (PAIR ? 2 : 1) * (it.t1 - it.t0);
+        const int nx = it.t1 - it.t0;
         for (int pass = 0; pass < 2 && !*abort; ++pass) {
           const CUtensorMap* tm = pass ? &tmV : &tmK;
           for (int x = 0; x < nx; ++x, ++g) {
-            const int j = it.t0 + (PAIR ? x >> 1 : x), rt = r + (PAIR ? x & 1 : 0);
+            const int j = it.t0 + x, rt = r;
             const int s = g % kStages;
             if (!mbar_wait(&bar[B_EMPTY + s], ((g / kStages) & 1) ^ 1, abort, p.dbg, 2u, (unsigned)g)) break;
             // the tile's tokens: all 128, or the row's ragged last tile, loaded
@@ -647,9 +586,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int qb = gr & 1;
         if (!mbar_wait(&bar[B_QFULL + qb], (gr >> 1) & 1, abort, p.dbg, 3u, (unsigned)gr)) break;
         tc_fence_after();
-        const int nx = (PAIR ? 2 : 1) * (it.t1 - it.t0);  // PAIR: the rows' tiles alternate
+        const int nx = it.t1 - it.t0;
         for (int x = 0; x < nx; ++x, ++g, ++gs) {
-          const uint32_t qlo = q_lo + (uint32_t)(PAIR ? 2 * qb + (x & 1) : qb) * (L::QBYTES >> 4);
+          const uint32_t qlo = q_lo + (uint32_t)qb * (L::QBYTES >> 4);
           const int s = g % kStages, b = gs & 1;
           if (!mbar_wait(&bar[B_FULL + s], (g / kStages) & 1, abort, p.dbg, 4u, (unsigned)g)) break;
           if (!mbar_wait(&bar[B_SEMPTY + b], ((gs >> 1) & 1) ^ 1, abort, p.dbg, 5u, (unsigned)gs)) break;
@@ -671,8 +610,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int x = 0; x < nx; ++x, ++g, ++gv) {
           const int s = g % kStages, pb = gv & 1;
           // the first tile of each row starts its accumulator
-          const bool first = PAIR ? x < 2 : x == 0;
-          const uint32_t ocol = kColO + (PAIR && (x & 1) ? (uint32_t)(kColOB - kColO) : 0u);
+          const bool first = x == 0;
+          const uint32_t ocol = kColO;
           if (!mbar_wait(&bar[B_FULL + s], (g / kStages) & 1, abort, p.dbg, 13u, (unsigned)g)) break;
           // only these MMAs read a V stage: the four epilogue arrivals of the
           // stage's release are made here (its last one is the commit below)
@@ -706,7 +645,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int gr = 0;; ++gr) {
         const Item it = read_item(items, gr, abort, p.dbg, 24u);
         if (it.row < 0) break;
-        const int nx = (PAIR ? 2 : 1) * (it.t1 - it.t0);
+        const int nx = it.t1 - it.t0;
         for (int x = 0; x < nx; ++x, ++gv) {
           const int pb = gv & 1;
           if (!mbar_wait(&bar[B_AFULL + pb], (gv >> 1) & 1, abort, p.dbg, 16u, (unsigned)gv)) break;
@@ -735,26 +674,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int etid = ew * 32 + lane;            // 0..255
     const uint32_t lane_addr = tmem + ((uint32_t)(quad * 32) << 16);
     const float c = p.c;
-    // the team that works on one row: both warpgroups, or (PAIR) one each
-    constexpr int kTeam = PAIR ? kEpi / 2 : kEpi;
-    const int tid = PAIR ? etid % kTeam : etid;    // thread within the team
-    const int w0 = PAIR ? wg * (kTeam / kWarp) : 0;  // the team's first epilogue warp
-    auto sync = [wg] {
-      if constexpr (PAIR) named_bar(2 + wg, kTeam);
-      else named_bar(1, kEpi);
-    };
-    const SelectScratch scr = (PAIR && wg == 1) ? SelectScratch{s_hist2, s_sh2, s_wsum2, s_best2, s_best_slot2}
-                                                : SelectScratch{s_hist, s_sh, s_wsum, s_best, s_best_slot};
-    // PAIR: this team's logits of head G-1, then scores
-    float* const scw = sc + (PAIR ? wg * kPairTok : 0);
-    // TMEM column of the stashed logits of this team's tile j
-    auto stash_at = [wg](int j) -> uint32_t {
-      if constexpr (PAIR) return (uint32_t)((wg ? kStashB : kPairStashA) + GS * j);
-      else return stash_col<G>(j);
-    };
-    // position of this team's tile j in the item's tile sequence
-    auto tpos = [wg](int j, int t0) { return PAIR ? 2 * j + wg : j - t0; };
-    constexpr int JS = PAIR ? 1 : 2;  // step between a team's tiles
+    constexpr int kTeam = kEpi;                 // both warpgroups work on a row
+    const int tid = etid;
+    constexpr int w0 = 0;
+    auto sync = [] { named_bar(1, kEpi); };
+    const SelectScratch scr{s_hist, s_sh, s_wsum, s_best, s_best_slot};
+    float* const scw = sc;  // logits of head G-1, then scores
+    // TMEM column of the stashed logits of tile j
+    auto stash_at = [](int j) -> uint32_t { return stash_col<G>(j); };
+    // position of tile j in the item's tile sequence
+    auto tpos = [](int j, int t0) { return j - t0; };
+    constexpr int JS = 2;  // step between a warpgroup's tiles
     int g = 0, gs = 0, gv = 0;
     for (int gr = 0;; ++gr) {
       int4 iv = make_int4(-1, 0, 0, 0);
@@ -768,8 +698,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       iv.w = __shfl_sync(0xffffffffu, iv.w, 0);
       if (named_bar_or(1, kEpi, *abort != 0 || iv.x < 0)) break;
       const Item it{iv.x, iv.y, iv.z, iv.w};
-      const int r = it.row + (PAIR ? wg : 0), t0 = it.t0, t1 = it.t1, nTi = it.t1 - it.t0;
-      const int nItem = (PAIR ? 2 : 1) * nTi;  // tiles of the item
+      const int r = it.row, t0 = it.t0, t1 = it.t1, nTi = it.t1 - it.t0;
+      const int nItem = nTi;  // tiles of the item
       // this row's length (after the append) and budget
       const int n = PERROW ? p.rowlen[r] : n_step;
       const int Bsel = PERROW ? (fs.B > 0 ? fs.B : p.rowbudget[r]) : fs.B;
@@ -815,7 +745,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int h = 0; h < G; ++h) { m[h] = kNoMax; l[h] = 0.f; u[h] = 0.f; }
 
       // ---------------- K pass: this warpgroup's tiles (global index parity)
-      for (int j = PAIR ? t0 : t0 + ((wg - gs) & 1); j < t1; j += JS) {
+      for (int j = t0 + ((wg - gs) & 1); j < t1; j += JS) {
         const int gj = g + tpos(j, t0), gsj = gs + tpos(j, t0);
         const int s = gj % kStages, b = gsj & 1;
         mbar_wait(&bar[B_SFULL + b], (gsj >> 1) & 1, abort, p.dbg, 6u, (unsigned)gsj);
@@ -870,7 +800,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // K pass), loaded two own tiles ahead: window sums (this thread wrote
       // them in the K pass), positions, |v|; the first two issued here, so that
       // their latency overlaps the statistics merge
-      const int j0 = PAIR ? t0 : t0 + ((wg - gv) & 1);
+      const int j0 = t0 + ((wg - gv) & 1);
       const float4* szrow = p.SZ + rbase + tok;
       const int* posrow = p.pos + rbase + tok;
       const float* vnrow = p.vnorm + rbase + tok;
@@ -982,19 +912,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int h = 0; h < G; ++h) {
         M[h] = Mm[h];
-        // H = ln l - ln 2 u / l. Whole rows take log2 l from the hardware log2
-        // and divide (l >= 1: the row's largest logit contributes 2^0), row
-        // pairs from log2f and logf: each measured the faster for its
-        // schedule (the kernel's speed on these shapes moves by several
-        // per cent with its code layout)
-        if constexpr (PAIR) {
-          NL[h] = -log2f(Ll[h]);
-          Hh[h] = logf(Ll[h]) - 0.69314718055994531f * (Uu[h] / Ll[h]);
-        } else {
-          const float lg = lg2_approx(Ll[h]);
-          NL[h] = -lg;
-          Hh[h] = 0.69314718055994531f * (lg - __fdividef(Uu[h], Ll[h]));
-        }
+        // H = ln l - ln 2 u / l, log2 l from the hardware log2 and the quotient
+        // from the hardware divide (l >= 1: the row's largest logit contributes 2^0)
+        const float lg = lg2_approx(Ll[h]);
+        NL[h] = -lg;
+        Hh[h] = 0.69314718055994531f * (lg - __fdividef(Uu[h], Ll[h]));
         if (tid == h) L0 = Ll[h];
       }
       // G = 8: the V pass reads the row's final statistics from shared memory
@@ -1242,12 +1164,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ---------------- attention output (warpgroup 0); a half row's two
       // partial sums (weights already normalised by the whole row) add up
       float ov[G];
-      if (PAIR || wg == 0) {
+      if (wg == 0) {
         mbar_wait(&bar[B_OFULL], gr & 1, abort, p.dbg, 11u, (unsigned)gr);
         __syncwarp();
         tc_fence_after();
         float o16[16];
-        tmem_ld16(lane_addr + (PAIR && wg ? kColOB : kColO), o16);
+        tmem_ld16(lane_addr + kColO, o16);
         tmem_ld_wait();
         tc_fence_before();
         __syncwarp();
@@ -1268,7 +1190,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         sync();
       }
-      if ((PAIR || wg == 0) && half <= 0 && tok < D && x_ok &&
+      if (wg == 0 && half <= 0 && tok < D && x_ok &&
           DC_INB(p, (long long)((r / p.kvh) * p.qh + (r % p.kvh) * G) * D + (G - 1) * D + tok,
                  (long long)(p.R / p.kvh) * p.qh * D, 115)) {
         float* op = fs.out + ((r / p.kvh) * p.qh + (r % p.kvh) * G) * D;
@@ -1303,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) { scr.best[tw] = bk; scr.best_slot[tw] = bs; scr.hist[tw] = bp; }
         sync();
         if (half < 0) {
-          // whole rows and row pairs: the warp that holds slot B reduces the
+          // whole rows: the warp that holds slot B reduces the
           // team's candidates itself (in warp order, as one thread would) and
           // fills the evicted slot; no further barrier (the candidates' next
           // writers are behind the next item's barriers)
@@ -1374,22 +1296,22 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 
 template <int D, int G, bool LONG, bool FULL = false, bool HEUR = false, bool GLOB = false, bool PERROW = false,
-          bool PAIR = false, bool GRAPH = false>
+          bool GRAPH = false>
 static cudaError_t launch_t(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                             const FusedPolicy& fp, int grid, cudaStream_t s) {
-  constexpr int kSmemBytes = Smem<PAIR, G>::BYTES;
+  constexpr int kSmemBytes = Smem<G>::BYTES;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, PAIR, GRAPH>,
+    cudaError_t e = cudaFuncSetAttribute(fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, GRAPH>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   if (fs.half_rows == 0 && !GRAPH)
-    return launch_pdl(fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, PAIR, GRAPH>, dim3(grid), dim3(kThreads),
+    return launch_pdl(fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, GRAPH>, dim3(grid), dim3(kThreads),
                       kSmemBytes, s, maps.k, maps.v, maps.k16, maps.v16, p, st, fs, fp);
   if (fs.half_rows == 0) {
-    fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, PAIR, GRAPH>
+    fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, GRAPH>
         <<<grid, kThreads, kSmemBytes, s>>>(maps.k, maps.v, maps.k16, maps.v16, p, st, fs, fp);
     return cudaGetLastError();
   }
@@ -1405,7 +1327,7 @@ static cudaError_t launch_t(const FusedMaps& maps, const Dev& p, const Step& st,
   la[0].val.cooperative = 1;
   cfg.attrs = la;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, PAIR, GRAPH>, maps.k, maps.v,
+  return cudaLaunchKernelEx(&cfg, fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, GRAPH>, maps.k, maps.v,
                             maps.k16, maps.v16, p, st, fs, fp);
 }
 
