@@ -314,24 +314,18 @@ dc_status dc_sync(dc_cache* h);
  *   q:   bf16 [rows][group][head_dim]; k, v: bf16 [rows][n][head_dim]
  *        (16-byte aligned); out: fp32 [rows][group][head_dim]; all device.
  *   stream: cudaStream_t (NULL: legacy default stream).
- * The split-K partial results go to a 16 MiB file-scope device array that
- * stays reserved, on every GPU where this library's device code is loaded,
- * until the process exits. With CUDA's lazy module loading (the default since
- * CUDA 12.2) that code, and so the array, is loaded on a device at the first
- * call there: a caller that reserves the rest of device memory up front must
- * make one call (a warm-up) on each device before it does, or that first call
- * can fail with DC_ERR_CUDA (out of memory while loading the module).
- * DC_ERR_CAPACITY if one split of all rows does not fit it, i.e. if
- * rows * group * (head_dim + 4) * 4 > 16 MiB; DC_ERR_INVALID_ARG for bad
- * shapes (head_dim 64 or 128, group 1, 2, 4 or 8, 1 <= rows <= 65535, n >= 1).
- * The first call on a device looks up the array's device address (once per
- * device, with that device current); make that first call before any stream
- * capture. Every call shares the array, which keeps the last call's
- * contents; nothing in it has to start at zero, because each call writes every
- * partial result before it reads it. Calls that overlap on the GPU (two
- * streams, or two host threads) race on the array and must be serialised by
- * the caller. Asynchronous on `stream`; dc_noalloc_last_error() describes a
- * failure. */
+ * The split-K partial results of a row merge through the shared memory of a
+ * thread-block cluster: the call has no device memory of its own. With CUDA's
+ * lazy module loading (the default since CUDA 12.2) the library's device code
+ * is loaded on a device at the first call there: a caller that reserves the
+ * rest of device memory up front must make one call (a warm-up) on each device
+ * before it does, or that first call can fail with DC_ERR_CUDA (out of memory
+ * while loading the module).
+ * DC_ERR_CAPACITY if rows * group * (head_dim + 4) * 4 > 16 MiB;
+ * DC_ERR_INVALID_ARG for bad shapes (head_dim 64 or 128, group 1, 2, 4 or 8,
+ * 1 <= rows <= 65535, n >= 1). Make the first call on a device before any
+ * stream capture. Calls may overlap on the GPU. Asynchronous on `stream`;
+ * dc_noalloc_last_error() describes a failure. */
 dc_status dc_attend_noalloc(const void* q, const void* k, const void* v, int rows, int n,
                             int head_dim, int group, float* out, void* stream);
 

@@ -969,12 +969,10 @@ dc_status dc_full_decode(dc_cache* h, const void* q, float* out) {
     if (e != cudaSuccess) return cuda_fail(h, e, "full decode");
     return launch_error(h, "full decode");
   }
-  int nsplit, chunk;
-  split_plan(h, h->n, &nsplit, &chunk);
   bool ok;
   {
-    Phase ph(h, DC_PHASE_FULL, 2);
-    ok = dc::launch_full_decode(h->dev, h->n, nsplit, chunk, q, out, h->stream);
+    Phase ph(h, DC_PHASE_FULL, 1);
+    ok = dc::launch_full_decode(h->dev, h->n, h->num_sms, q, out, h->stream);
   }
   if (!ok) return fail(h, DC_ERR_INVALID_ARG, "unsupported head_dim / group");
   return launch_error(h, "full decode");

@@ -34,7 +34,8 @@ void launch_glob_evict(const Dev& p, int n, int B, cudaStream_t s);
 // [nrows][cap].
 void launch_convert_sz(const Dev& p, int row0, int nrows, int which, double* dst, cudaStream_t s);
 
-bool launch_full_decode(const Dev& p, int n, int nsplit, int chunk, const void* q, float* out,
-                        cudaStream_t s);
+// Full-cache decode attention on CUDA cores over the first n tokens of every row
+// (Dev: R, stride, d, G, qh, kvh, K, V, c).
+bool launch_full_decode(const Dev& p, int n, int num_sms, const void* q, float* out, cudaStream_t s);
 
 }  // namespace dc
