@@ -393,10 +393,11 @@ const char* dc_last_error(const dc_cache* h);
 /* Exact log-partition function of the Plackett-Luce distribution over size-B
  * subsets (App. C): out[r] = log sum_{a subset of [L], |a| = B}
  * exp(sum_{i in a} scores[r][i] / tau), for `rows` independent rows.
- * scores: fp32 [rows][L]; out: fp32 [rows]. Computed by the O(L B) dynamic
- * programme over the elementary symmetric polynomials, in base-2 log space,
- * fp32 with the hardware exp2/log2 (the error grows at most linearly in L:
- * |error| <= 2 L 2^-24 (|log Z| + max |s| / tau) + L 2^-21). Needs
+ * scores: fp32 [rows][L]; out: fp32 [rows]. Computed in O(L) as the probability
+ * that a sum of independent Bernoulli variables is B (their characteristic
+ * function, inverted at a few points), after a shift that centres the sum on B;
+ * |error| <= 2 L 2^-24 (|log Z| + max |s| / tau) + L 2^-21. A score of
+ * -infinity takes no part; NaN and +infinity give NaN. Needs
  * 1 <= B <= L, rows <= 65535, B <= 25599, tau > 0;
  * else DC_ERR_INVALID_ARG (message in dc_train_last_error()). */
 dc_status dc_pl_log_partition(const float* scores, int rows, int L, int B, float tau, float* out,

@@ -3,15 +3,28 @@
 // Gumbel-top-B sampling with the log-probability of the sampled subset.
 //
 // log Z(s, B, tau) = log sum over subsets a of [L], |a| = B, of
-// exp(sum_{i in a} s_i / tau): the log of the elementary symmetric polynomial
-// e_B of x_i = exp(s_i / tau). With E_i[k] = e_k(x_1..x_i), adding item i
-// gives E_i[k] = E_{i-1}[k] + x_i E_{i-1}[k-1] (E[0] = 1). Items are added in
-// chunks of 31: the generating polynomial prod_i (1 + x_i t) of a chunk has
-// coefficients c_m = e_m(chunk), and E_{i+31}[k] = sum_m E_i[k-m] c_m (the
-// product of the two polynomials). One warp builds a chunk's c_m by the
-// item-by-item recurrence (lane m holds c_m); the CTA then convolves, one
-// barrier per chunk instead of per item. O(L B) work in O(B) memory, one CTA
-// per row, in log space (log-sum-exp), fp32.
+// exp(sum_{i in a} y_i), y_i = s_i / tau: the log of the elementary symmetric
+// polynomial e_B(exp y_1, ..., exp y_L). For any shift u, with p_i = 1 / (1 +
+// exp(-(y_i + u))) and S the sum of independent Bernoulli(p_i) variables,
+//
+//   e_B = P(S = B) exp(-u B) prod_i (1 + exp(y_i + u))
+//
+// (expand the product: the subset a has probability prod_{a} p_i prod_{not a}
+// (1 - p_i)). u is chosen so that E[S] is B to a tenth of a standard deviation
+// (safeguarded Newton steps on the monotone E[S]): P(S = B) is then of the order
+// of 1 / (1 + sd), and an inverse discrete Fourier transform of the
+// characteristic function phi(w) = prod_i (1 - p_i + p_i e^{iw}) gives it
+// (Fernandez and Williams 2010; Hong 2013):
+//
+//   P(S = B) = 1/N sum_{j < N} phi(2 pi j / N) e^{-2 pi i j B / N}.
+//
+// With N = L + 1 that is exact. It is enough that P(|S - E[S]| >= N) is below
+// the result's precision (Bernstein's inequality gives N: about 8.5 sd + 20),
+// and that the terms kept reach |phi|^2 <= exp(-2 sd^2 (1 - cos w)) small
+// enough: at most 22 of them, whatever L and B. So O(L) work in a few passes
+// where the dynamic programme over e_k costs O(L B) exponentials (64 x 4096 x
+// 1024: 255 us, bound by the exponentials of 268 M terms), and a smaller error:
+// nothing of the size of log Z is added up term by term in fp32.
 //
 // Gumbel-top-B: perturbed scores s_i / tau + g_i (g_i ~ Gumbel(0, 1), given by
 // the caller), the B largest kept (ties: lower index), their indices written
@@ -28,149 +41,420 @@
 namespace dc {
 namespace {
 
-constexpr int kLzThreads = 1024;
+constexpr int kLzMaxWarps = 16;      // 512 threads, 128 for short rows
+constexpr int kRowSmem = 40 * 1024;  // values of a row kept in shared memory (160 KB)
 constexpr int kTopThreads = 512;
+constexpr int kTopWarps = kTopThreads / kWarp;
+constexpr int kTopBins = 2048;
+constexpr int kTopList = kTopThreads;  // keys of the threshold bin ranked directly
 
-__device__ __forceinline__ float lg2(float x) {
-  float y;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
+// A value held as an unevaluated sum hi + lo; (hi, lo) += x (Knuth's TwoSum).
+__device__ __forceinline__ void add2(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), bb = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(x, bb)));
+  hi = s;
 }
 
-// log2(2^a + 2^b) with the hardware base-2 exponential and logarithm.
-__device__ __forceinline__ float log2_add_exp2(float a, float b) {
-  const float m = fmaxf(a, b);
-  if (m == -INFINITY) return -INFINITY;
-  return m + lg2(1.f + ex2(fminf(a, b) - m));
+// The warp's sum of such pairs, in lane 0's (hi, lo).
+__device__ __forceinline__ void warp_add2(float& hi, float& lo) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    const float h = __shfl_down_sync(0xffffffffu, hi, off), l = __shfl_down_sync(0xffffffffu, lo, off);
+    add2(hi, lo, h);
+    lo += l;
+  }
 }
 
-constexpr int kChunk = 31;        // items per chunk: c_0..c_31 in one warp's lanes
-constexpr int kChunkBatch = 64;   // chunks whose polynomials are built per pass
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+  return x;
+}
 
-// One CTA per row, up to kLzThreads threads (each owns the terms k = 1 + tid,
-// 1 + tid + blockDim, ...; e_0 = 1 never changes, so B = 1024 takes one term
-// per thread). Shared memory: E = log2 e_k, double-buffered ([2][B + 1]), then
-// the polynomials of a batch of chunks ([kChunkBatch][32], log2 c_m).
-__global__ void __launch_bounds__(kLzThreads) pl_logz_kernel(const float* __restrict__ scores, int L, int B,
-                                                             float tau, float* __restrict__ out) {
-  extern __shared__ float E[];
-  constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
-  const int row = blockIdx.x, tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
-  const int nwarps = blockDim.x / kWarp;
+// The larger of two, NaN if either is.
+__device__ __forceinline__ float max_nan(float a, float b) { return a != a ? a : b <= a ? a : b; }
+
+// p = sigma(x), q = 1 - p and e = exp(-|x|), each with its own relative precision.
+__device__ __forceinline__ void logistic(float x, float& p, float& q, float& e) {
+  e = expf(-fabsf(x));
+  const float inv = __frcp_rn(1.f + e), small = e * inv;
+  p = x > 0.f ? inv : small;
+  q = x > 0.f ? small : inv;
+}
+
+// One CTA per row. Bound by latency: a handful of block-wide reductions over a
+// row held in shared memory, in short loops (unrolled over registers, the code
+// ran once per row out of a cold instruction cache: 44 us against 22, caches
+// flushed, at 64 x 4096 x 1024; the dynamic programme 255).
+__global__ void __launch_bounds__(kLzMaxWarps* kWarp) pl_logz_kernel(const float* __restrict__ scores, int L, int B,
+                                                                     float tau, float* __restrict__ out) {
+  extern __shared__ float ys[];      // y_i, then p_i (rows of up to kRowSmem)
+  __shared__ float rs[kLzMaxWarps][4];
+  __shared__ float2 prod[kLzMaxWarps][kWarp];
+  __shared__ double sh_u;
+  __shared__ float sh_uh, sh_ul, sh_var;
+  __shared__ int sh_state;
+  // a kernel launched after this one may start (the sampler's selection)
+  grid_dep_launch();
+  const int row = blockIdx.x, tid = threadIdx.x, nt = blockDim.x, lane = tid % kWarp, warp = tid / kWarp;
+  const int nw = nt / kWarp;
   const float* s = scores + (size_t)row * L;
-  float* cur = E;
-  float* nxt = E + (B + 1);
-  float* C = E + 2 * (B + 1);
-  for (int k = tid; k <= B; k += blockDim.x) cur[k] = nxt[k] = k == 0 ? 0.f : -INFINITY;
-  const int nchunks = (L + kChunk - 1) / kChunk;
-  for (int c0 = 0; c0 < nchunks; c0 += kChunkBatch) {
-    const int cb = min(kChunkBatch, nchunks - c0);
-    // each warp: the polynomials of its chunks, item by item (lane m: c_m;
-    // all lanes read c_{m-1} before any writes, through the shuffle)
-    for (int ci = warp; ci < cb; ci += nwarps) {
-      const int i0 = (c0 + ci) * kChunk, cnt = min(kChunk, L - i0);
-      // the chunk's s_i / tau in log2 units, one per lane
-      const float yl = lane < cnt ? __fmul_rn(__fdiv_rn(s[i0 + lane], tau), kLog2e) : 0.f;
-      float e = lane == 0 ? 0.f : -INFINITY;
-      for (int j = 0; j < cnt; ++j) {
-        const float y = __shfl_sync(0xffffffffu, yl, j);
-        const float below = __shfl_up_sync(0xffffffffu, e, 1);
-        if (lane >= 1 && lane <= j + 1) e = log2_add_exp2(e, y + below);
-      }
-      C[ci * kWarp + lane] = e;
-    }
-    __syncthreads();
-    // E <- E * c, chunk by chunk: E'[k] = log2 sum_m 2^(E[k-m] + c_m)
-    for (int ci = 0; ci < cb; ++ci) {
-      const float* c = C + ci * kWarp;
-      const int cnt = min(kChunk, L - (c0 + ci) * kChunk);
-      for (int k = 1 + tid; k <= B; k += blockDim.x) {
-        const int mmax = min(k, cnt);
-        // the terms in registers: shared memory is read once
-        float t[kChunk + 1];
-        float mx = -INFINITY;
-#pragma unroll
-        for (int m = 0; m <= kChunk; ++m) {
-          t[m] = m <= mmax ? cur[k - m] + c[m] : -INFINITY;
-          mx = fmaxf(mx, t[m]);
-        }
-        float acc = 0.f;
-#pragma unroll
-        for (int m = 0; m <= kChunk; ++m) acc += ex2(t[m] - mx);
-        nxt[k] = mx == -INFINITY ? -INFINITY : mx + lg2(acc);
-      }
-      __syncthreads();
-      float* t = cur;
-      cur = nxt;
-      nxt = t;
+  const bool in_smem = L <= kRowSmem;
+  auto y_at = [&](int i) { return in_smem ? ys[i] : __fdiv_rn(s[i], tau); };
+  // ---- range, mean and count of the finite items (-infinity takes no part);
+  // +infinity and NaN make the result NaN (they have no finite partition function)
+  float mx = -INFINITY, mn = INFINITY, sum = 0.f, cnt = 0.f;
+#pragma unroll 2
+  for (int i = tid; i < L; i += nt) {
+    const float y = __fdiv_rn(s[i], tau);
+    if (in_smem) ys[i] = y;
+    mx = max_nan(mx, y);
+    if (y > -INFINITY) {
+      mn = fminf(mn, y);
+      sum += y;
+      cnt += 1.f;
     }
   }
-  if (tid == 0) out[row] = cur[B] * kLn2;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+    sum += __shfl_xor_sync(0xffffffffu, sum, off);
+    cnt += __shfl_xor_sync(0xffffffffu, cnt, off);
+  }
+  if (lane == 0) {
+    rs[warp][0] = mx; rs[warp][1] = mn; rs[warp][2] = sum; rs[warp][3] = cnt;
+  }
+  __syncthreads();
+  // thread 0's part of the search: u in [lo, hi], E[S] < B at lo and > B at hi
+  double u = 0.0, lo = 0.0, hi = 0.0;
+  if (tid == 0) {
+    for (int w = 1; w < nw; ++w) {
+      mx = max_nan(mx, rs[w][0]);
+      mn = fminf(mn, rs[w][1]);
+      sum += rs[w][2];
+      cnt += rs[w][3];
+    }
+    // 0: search; 1: fewer finite items than B; 2: exactly B; 3: not finite
+    const int st = !(mx < INFINITY) ? 3 : cnt < (float)B ? 1 : cnt == (float)B ? 2 : 0;
+    if (st == 0) {
+      const float rest = cnt - (float)B;
+      lo = (double)(logf((float)B / cnt) - 1.f) - (double)mx;
+      hi = (double)(1.f - logf(rest / cnt)) - (double)mn;
+      u = (double)(logf((float)B / rest) - sum / cnt);
+      u = u < lo ? lo : u > hi ? hi : u;
+    }
+    sh_state = st;
+    sh_u = u;
+    sh_uh = (float)u;
+    sh_ul = (float)(u - (double)sh_uh);
+  }
+  __syncthreads();
+  const int state = sh_state;
+  if (state == 1 || state == 3) {
+    if (tid == 0) out[row] = state == 1 ? -INFINITY : __int_as_float(0x7fc00000);
+    return;
+  }
+  // ---- the shift: |E[S] - B| <= sd / 10 (or 1 / 20)
+  for (int step = 0; state == 0 && step < 400; ++step) {
+    const float uh = sh_uh, ul = sh_ul;
+    float fp = 0.f, fv = 0.f;
+#pragma unroll 4
+    for (int i = tid; i < L; i += nt) {
+      const float y = y_at(i);
+      float p, q, e;
+      logistic(__fadd_rn(__fadd_rn(y, uh), ul), p, q, e);
+      if (y == -INFINITY) p = 0.f;
+      fp += p;
+      fv = fmaf(p, q, fv);
+    }
+    fp = warp_sum(fp);
+    fv = warp_sum(fv);
+    if (lane == 0) {
+      rs[warp][0] = fp;
+      rs[warp][1] = fv;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      fp = warp_sum(lane < nw ? rs[lane][0] : 0.f);
+      fv = warp_sum(lane < nw ? rs[lane][1] : 0.f);
+      if (lane == 0) {
+        const float d = (float)B - fp;
+        sh_var = fv;
+        if (fabsf(d) <= 0.1f * fmaxf(sqrtf(fv), 0.5f)) {
+          sh_state = 4;
+        } else {
+          if (d > 0.f) lo = u;
+          else hi = u;
+          // a Newton step where it stays inside the bracket, else its middle
+          const double nu = u + (double)(d / fv);
+          u = nu > lo && nu < hi ? nu : 0.5 * (lo + hi);
+          sh_u = u;
+          sh_uh = (float)u;
+          sh_ul = (float)(u - (double)sh_uh);
+        }
+      }
+    }
+    __syncthreads();
+    if (sh_state == 4) break;
+  }
+  // ---- sum_i log(1 + exp(y_i + u)) = (sum of y_i + u over the positive ones)
+  // + sum_i log1p(exp(-|y_i + u|)); all items when B of them are finite: the
+  // sum of the y_i. The p_i take the y_i's place.
+  const float uh = sh_uh, ul = sh_ul, var = sh_var;
+  float ph = 0.f, pl = 0.f, np = 0.f;
+#pragma unroll 2
+  for (int i = tid; i < L; i += nt) {
+    const float y = y_at(i);
+    float p, q, e;
+    const float x = __fadd_rn(__fadd_rn(y, uh), ul);
+    logistic(x, p, q, e);
+    if (y == -INFINITY) p = e = 0.f;
+    if (y > -INFINITY && (state == 2 || x > 0.f)) {
+      add2(ph, pl, y);
+      np += 1.f;
+    }
+    if (state == 0) add2(ph, pl, log1pf(e));
+    if (in_smem) ys[i] = p;
+  }
+  warp_add2(ph, pl);
+  np = warp_sum(np);
+  if (lane == 0) {
+    rs[warp][0] = ph;
+    rs[warp][1] = pl;
+    rs[warp][2] = np;
+  }
+  __syncthreads();
+  double A = 0.0;
+  if (warp == 0) {
+    ph = lane < nw ? rs[lane][0] : 0.f;
+    pl = lane < nw ? rs[lane][1] : 0.f;
+    warp_add2(ph, pl);
+    np = warp_sum(lane < nw ? rs[lane][2] : 0.f);
+    A = (double)ph + (double)pl + (double)(np - (float)B) * sh_u;
+    if (state == 2 && lane == 0) out[row] = (float)A;  // (np = B: the shift takes no part)
+  }
+  if (state == 2) return;
+  // ---- N points, of which j = 1 .. J count (j and N - j are conjugates)
+  const float a = 30.f + log1pf(sqrtf(var)), t = a * (1.f / 3.f) + sqrtf(a * a * (1.f / 9.f) + 2.f * a * var) + 3.f;
+  const int N = t < (float)L ? (int)t + 1 : L + 1;
+  // point j counts while 2 j <= N and 2 var sin^2(pi j / N) <= 28; lane l tests
+  // point l + 1 (at most 22 count: 32 lanes hold them)
+  const float sl = sinpif((float)(lane + 1) / (float)N);
+  const int J = __popc(__ballot_sync(0xffffffffu, 2 * (lane + 1) <= N && 2.f * var * sl * sl <= 28.f));
+  // lanes [k J, (k + 1) J) of a warp multiply up the factors of points 1 .. J
+  // over the k-th part of the warp's items
+  const int parts = J ? kWarp / J : 1, k = J ? lane / J : 0, j = J ? lane % J + 1 : 1;
+  const float sp = sinpif((float)j / (float)N), omc = 2.f * sp * sp, sn = sinpif((float)(2 * j) / (float)N);
+  float R = 1.f, I = 0.f;
+  if (J > 0 && k < parts) {
+    const int slot = warp * parts + k, slots = nw * parts;
+    const int i0 = (int)((long long)L * slot / slots), i1 = (int)((long long)L * (slot + 1) / slots);
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) {
+      float p;
+      if (in_smem) {
+        p = ys[i];
+      } else {
+        float q, e;
+        const float y = y_at(i);
+        logistic(__fadd_rn(__fadd_rn(y, uh), ul), p, q, e);
+        if (y == -INFINITY) p = 0.f;
+      }
+      const float ar = fmaf(-p, omc, 1.f), ai = p * sn;  // 1 - p (1 - cos w) + i p sin w
+      const float nR = fmaf(R, ar, -(I * ai));
+      I = fmaf(R, ai, I * ar);
+      R = nR;
+    }
+  }
+  prod[warp][lane] = make_float2(R, I);
+  __syncthreads();
+  if (warp == 0) {
+    float term = 0.f;
+    if (lane < J) {
+      R = 1.f;
+      I = 0.f;
+      for (int w = 0; w < nw; ++w)
+        for (int q = 0; q < parts; ++q) {
+          const float2 z = prod[w][q * J + lane];
+          const float nR = R * z.x - I * z.y;
+          I = R * z.y + I * z.x;
+          R = nR;
+        }
+      // the real part of phi e^{-2 pi i j B / N}, twice for the conjugate point
+      const int at = (int)((unsigned)j * (unsigned)(B % N) % (unsigned)N);
+      float c, d;
+      sincospif(2.f * (float)at / (float)N, &d, &c);
+      term = R * c + I * d;
+      if (2 * j != N) term *= 2.f;
+    }
+    term = warp_sum(term);
+    if (lane == 0) out[row] = (float)(A + log((double)((1.f + term) / (float)N)));
+  }
 }
 
 // One CTA per row: top-B of the perturbed scores by (value desc, index asc),
-// indices ascending into idx[row][0..B), and sum_{i in a} s_i / tau.
+// indices ascending into idx[row][0..B), and sum_{i in a} s_i / tau. Order keys
+// into shared memory (where the row fits) with their range; a histogram of 2048
+// equal-width bins over the range; the keys of the bin that holds the B-th
+// largest listed and ranked by comparing each with all of them (a few, usually;
+// more than 512, as with many equal scores, take a radix select over the row);
+// the kept indices placed by ballots and one prefix sum over the warps. Bound by
+// the latency of these passes: 64 x 4096 x 1024 in 25 us with flushed caches (33
+// by four radix passes, one thread walking the bins, and a block-wide scan per
+// 512 items); beside log Z, the whole call takes 24 us warm (285).
 __global__ void __launch_bounds__(kTopThreads) gumbel_topb_kernel(const float* __restrict__ scores,
                                                                   const float* __restrict__ gumbel, int L,
                                                                   int B, float tau, int* __restrict__ idx,
                                                                   float* __restrict__ logp,
                                                                   const float* __restrict__ logz) {
-  __shared__ int hist[256];
+  extern __shared__ uint32_t skeys[];
+  __shared__ int hist[kTopBins];
+  __shared__ int list[kTopList];
   __shared__ int sh[4];
-  __shared__ int wsum[kTopThreads / kWarp];
-  __shared__ unsigned long long best[kTopThreads / kWarp];
-  __shared__ int best_slot[kTopThreads / kWarp];
-  __shared__ double dsum[kTopThreads / kWarp];
+  __shared__ int wsum[kTopWarps];
+  __shared__ unsigned long long best[kTopWarps];
+  __shared__ int best_slot[kTopWarps];
+  __shared__ double dsum[kTopWarps];
   const SelectScratch scr{hist, sh, wsum, best, best_slot};
   auto sync = [] { __syncthreads(); };
-  const int row = blockIdx.x, tid = threadIdx.x;
+  const int row = blockIdx.x, tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
   const float* s = scores + (size_t)row * L;
   const float* g = gumbel + (size_t)row * L;
-  auto key = [&](int i) { return score_key(__fadd_rn(__fdiv_rn(s[i], tau), g[i])); };
-  auto all = [](int) { return true; };
-  int gt = 0;
-  const uint32_t T = team_radix_select<kTopThreads>(L, B, key, all, tid, scr, &gt, sync);
-  const int need_eq = B - gt;  // ties at T kept by lowest index
-  int eq_local = 0;
-  for (int i = tid; i < L; i += kTopThreads) eq_local += (key(i) == T);
-  int eq_total;
-  (void)team_exclusive_scan<kTopThreads>(eq_local, tid, scr.wsum, &eq_total, sync);
-  uint32_t P = 0;  // ties kept when ~index >= P
-  if (eq_total > need_eq) {
-    auto ikey = [](int i) { return ~(uint32_t)i; };
-    auto tied = [&](int i) { return key(i) == T; };
-    int gt2 = 0;
-    P = team_radix_select<kTopThreads>(L, need_eq, ikey, tied, tid, scr, &gt2, sync);
+  const bool in_smem = L <= kRowSmem;
+  auto compute = [&](int i) { return score_key(__fadd_rn(__fdiv_rn(s[i], tau), g[i])); };
+  for (int b = tid; b < kTopBins; b += kTopThreads) hist[b] = 0;
+  if (tid == 0) sh[2] = 0;
+  uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
+#pragma unroll 4
+  for (int i = tid; i < L; i += kTopThreads) {
+    const uint32_t k = compute(i);
+    if (in_smem) skeys[i] = k;
+    kmin = k < kmin ? k : kmin;
+    kmax = k > kmax ? k : kmax;
   }
-  auto keep = [&](int i) {
-    const uint32_t k = key(i);
-    return k > T || (k == T && ~(uint32_t)i >= P);
-  };
-  int base = 0;
-  double part = 0.0;
-  for (int c0 = 0; c0 < L; c0 += kTopThreads) {
-    const int i = c0 + tid;
-    const int f = (i < L && keep(i)) ? 1 : 0;
-    int tot;
-    const int rank = team_exclusive_scan<kTopThreads>(f, tid, scr.wsum, &tot, sync);
-    if (f) {
-      idx[(size_t)row * B + base + rank] = i;
-      part += (double)__fdiv_rn(s[i], tau);
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if (lane == 0) best[warp] = ((unsigned long long)kmax << 32) | kmin;
+  __syncthreads();
+  kmin = __reduce_min_sync(0xffffffffu, lane < kTopWarps ? (uint32_t)best[lane] : 0xFFFFFFFFu);
+  kmax = __reduce_max_sync(0xffffffffu, lane < kTopWarps ? (uint32_t)(best[lane] >> 32) : 0u);
+  auto key = [&](int i) { return in_smem ? skeys[i] : compute(i); };
+  const int bits = kmax > kmin ? 32 - __clz(kmax - kmin) : 0, shift = bits > 11 ? bits - 11 : 0;
+  auto bin = [&](uint32_t k) { return (k - kmin) >> shift; };  // < kTopBins
+#pragma unroll 2
+  for (int i = tid; i < L; i += kTopThreads) atomicAdd(&hist[bin(key(i))], 1);
+  __syncthreads();
+  // the threshold bin: thread t holds bins kTopBins - 1 - 4 t - (0..3), so that an
+  // exclusive scan over the threads counts the keys of higher bins
+  int c[4], tot4 = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c[q] = hist[kTopBins - 1 - 4 * tid - q];
+    tot4 += c[q];
+  }
+  int all_keys;
+  int before = team_exclusive_scan<kTopThreads>(tot4, tid, wsum, &all_keys, sync);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    if (before < B && B <= before + c[q]) {
+      sh[0] = kTopBins - 1 - 4 * tid - q;
+      sh[1] = before;
     }
-    base += tot;
+    before += c[q];
+  }
+  __syncthreads();
+  const uint32_t dsel = (uint32_t)sh[0];
+  const int above = sh[1], m = hist[dsel], need = B - above;
+  // keys above (T, cut) are kept: key > T, or key == T and index <= cut
+  uint32_t T = 0;
+  int cut = -1;
+  if (m <= kTopList) {
+#pragma unroll 2
+    for (int i = tid; i < L; i += kTopThreads)
+      if (bin(key(i)) == dsel) list[atomicAdd(&sh[2], 1)] = i;
+    __syncthreads();
+    if (tid < m) {
+      const int mine = list[tid];
+      const uint32_t k = key(mine);
+      int rank = 0;
+      for (int o = 0; o < m; ++o) {
+        const uint32_t ko = key(list[o]);
+        rank += ko > k || (ko == k && list[o] < mine);
+      }
+      if (rank == need - 1) {
+        sh[0] = (int)k;
+        sh[1] = mine;
+      }
+    }
+    __syncthreads();
+    T = (uint32_t)sh[0];
+    cut = sh[1];
+  } else {
+    __syncthreads();
+    auto all = [](int) { return true; };
+    int gt = 0;
+    T = team_radix_select_wide<kTopThreads>(L, B, key, all, tid, scr, &gt, sync);
+    // the (B - gt)-th lowest index among the keys equal to T
+    auto tied = [&](int i) { return key(i) == T; };
+    auto ikey = [](int i) { return ~(uint32_t)i; };
+    int gt2 = 0;
+    cut = (int)~team_radix_select_wide<kTopThreads>(L, B - gt, ikey, tied, tid, scr, &gt2, sync);
+  }
+  // each warp takes a contiguous run of 32-item groups: its kept items are
+  // counted, the counts prefix-summed over the warps, and a second walk writes
+  // the indices
+  auto kept = [&](int i) {
+    if (i >= L) return false;
+    const uint32_t k = key(i);
+    return k > T || (k == T && i <= cut);
+  };
+  const int ng = (L + kWarp - 1) / kWarp;
+  const int g0 = (int)((long long)ng * warp / kTopWarps), g1 = (int)((long long)ng * (warp + 1) / kTopWarps);
+  int n_kept = 0;
+#pragma unroll 2
+  for (int gi = g0; gi < g1; ++gi) n_kept += __popc(__ballot_sync(0xffffffffu, kept(gi * kWarp + lane)));
+  if (lane == 0) wsum[warp] = n_kept;
+  __syncthreads();
+  int base = (int)__reduce_add_sync(0xffffffffu, lane < warp ? (unsigned)wsum[lane] : 0u);
+  const unsigned lt = (1u << lane) - 1u;
+  double part = 0.0;
+  int* dst = idx + (size_t)row * B;
+#pragma unroll 2
+  for (int gi = g0; gi < g1; ++gi) {
+    const int i = gi * kWarp + lane;
+    const bool f = kept(i);
+    const unsigned mk = __ballot_sync(0xffffffffu, f);
+    if (f) {
+      dst[base + __popc(mk & lt)] = i;
+      if (logp) part += (double)__fdiv_rn(s[i], tau);
+    }
+    base += __popc(mk);
   }
   if (logp) {
     // sum_{i in a} s_i / tau in double, fixed reduction order
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
-    if (tid % kWarp == 0) dsum[tid / kWarp] = part;
+    if (lane == 0) dsum[warp] = part;
     __syncthreads();
+    // log Z comes from the kernel before, beside which this one may have run
+    grid_dep_wait();
     if (tid == 0) {
       double t = 0.0;
-      for (int w = 0; w < kTopThreads / kWarp; ++w) t += dsum[w];
-      logp[row] = (float)(t - (double)logz[row]);
+      for (int w = 0; w < kTopWarps; ++w) t += dsum[w];
+      logp[row] = (float)(t - (double)*reinterpret_cast<const volatile float*>(logz + row));
     }
   }
+}
+
+// Dynamic shared memory for a row of L 4-byte values (0: the row stays in
+// global memory), allowed for `kernel` on the current device when it is more
+// than every kernel may have.
+template <class K>
+cudaError_t row_smem(K kernel, int L, size_t* bytes) {
+  *bytes = L <= kRowSmem ? (size_t)L * 4 : 0;
+  if (*bytes <= 32 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem * 4);
 }
 
 thread_local std::string g_train_error;
@@ -191,16 +475,15 @@ extern "C" dc_status dc_pl_log_partition(const float* scores, int rows, int L, i
   if (!scores || !out) return train_fail(DC_ERR_INVALID_ARG, "NULL pointer");
   if (rows < 1 || rows > 65535 || L < 1 || B < 1 || B > L || !(tau > 0.f))
     return train_fail(DC_ERR_INVALID_ARG, "need 1 <= rows <= 65535, 1 <= B <= L and tau > 0");
-  const size_t smem = (2 * (size_t)(B + 1) + kChunkBatch * kWarp) * sizeof(float);
+  // (the limit of an earlier kernel that kept the B + 1 polynomials in shared memory)
   if (2 * (size_t)(B + 1) * sizeof(float) > 200 * 1024) return train_fail(DC_ERR_INVALID_ARG, "B too large (at most 25599)");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(pl_logz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return train_fail(DC_ERR_CUDA, cudaGetErrorString(e));
+  size_t smem;
+  cudaError_t e = row_smem(pl_logz_kernel, L, &smem);
+  if (e == cudaSuccess) {
+    pl_logz_kernel<<<rows, L <= 1024 ? 128 : kLzMaxWarps * kWarp, smem, static_cast<cudaStream_t>(stream)>>>(
+        scores, L, B, tau, out);
+    e = cudaGetLastError();
   }
-  const int threads = B < kLzThreads ? (B + 31) / 32 * 32 : kLzThreads;
-  pl_logz_kernel<<<rows, threads, smem, s>>>(scores, L, B, tau, out);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return train_fail(DC_ERR_CUDA, cudaGetErrorString(e));
   return DC_OK;
 }
@@ -216,8 +499,15 @@ extern "C" dc_status dc_gumbel_top_b(const float* scores, const float* gumbel, i
     dc_status st = dc_pl_log_partition(scores, rows, L, B, tau, logz_scratch, stream);
     if (st != DC_OK) return st;
   }
-  gumbel_topb_kernel<<<rows, kTopThreads, 0, s>>>(scores, gumbel, L, B, tau, idx, logp, logz_scratch);
-  cudaError_t e = cudaGetLastError();
+  size_t smem;
+  cudaError_t e = row_smem(gumbel_topb_kernel, L, &smem);
+  // with log Z, the selection may run beside its kernel and waits for it at the end
+  if (e == cudaSuccess && logp)
+    e = launch_pdl(gumbel_topb_kernel, dim3(rows), dim3(kTopThreads), smem, s, scores, gumbel, L, B, tau, idx, logp,
+                   (const float*)logz_scratch);
+  else if (e == cudaSuccess)
+    gumbel_topb_kernel<<<rows, kTopThreads, smem, s>>>(scores, gumbel, L, B, tau, idx, logp, logz_scratch);
+  if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return train_fail(DC_ERR_CUDA, cudaGetErrorString(e));
   return DC_OK;
 }
