@@ -921,7 +921,7 @@ dc_status dc_evict(dc_cache* h, int budget) {
   if (h->per_row) {
     // every row to its own budget (or all to `budget` when > 0)
     {
-      Phase ph(h, DC_PHASE_EVICT, dc::evict_kernel_count(h->n, budget > 0 ? budget : 0));
+      Phase ph(h, DC_PHASE_EVICT, dc::evict_kernel_count(h->dev, h->n, budget > 0 ? budget : 0));
       dc::launch_evict(h->dev, h->n, budget > 0 ? budget : 0, h->stream);
     }
     dc_status s = launch_error(h, "evict");
@@ -938,7 +938,7 @@ dc_status dc_evict(dc_cache* h, int budget) {
   const int B = effective_budget(h, budget, h->n, h->seen);
   const int keep = std::min(h->n, B);
   if (keep < h->n) {
-    Phase ph(h, DC_PHASE_EVICT, h->dev.seq_rows ? 2 : dc::evict_kernel_count(h->n, keep));
+    Phase ph(h, DC_PHASE_EVICT, h->dev.seq_rows ? 2 : dc::evict_kernel_count(h->dev, h->n, keep));
     if (h->dev.seq_rows) dc::launch_glob_evict(h->dev, h->n, keep, h->stream);
     else dc::launch_evict(h->dev, h->n, keep, h->stream);
     dc_status s = launch_error(h, "evict");

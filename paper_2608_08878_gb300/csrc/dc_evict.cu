@@ -207,13 +207,82 @@ __global__ void __launch_bounds__(kMoveThreads) evict_move_kernel(Dev p) {
   warp_move_batch(p, base, p.holes + base, p.holes + base + nh, k0, nmv, threadIdx.x % kWarp);
 }
 
+// One eviction from every row (the steady state, n == B + 1): the lowest-ranked
+// token is an argmin, and slot B (the last) the only slot that can move. One
+// CTA of 256 threads per row: slot B is loaded first, the scores with 16-byte
+// loads (at most a few per thread), the candidates reduced by redux (key, then
+// position among equal keys only) instead of the select kernel's keys in shared
+// memory and 32-way serial merges, and no move kernel after it. Bound by the
+// latency of three dependent loads: 256 rows x 1639 tokens 17.5 us (select and
+// an idle move kernel, caches flushed) -> 5.6 us.
+constexpr int kOneThreads = 256;
+
+__global__ void __launch_bounds__(kOneThreads) evict_one_kernel(Dev p, int n, int B) {
+  __shared__ uint32_t bkey[kOneThreads / kWarp];
+  __shared__ int bslot[kOneThreads / kWarp];
+  const int r = blockIdx.x, tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
+  const size_t base = (size_t)r * p.stride;
+  const int* ps = p.pos + base;
+  SlotCopy mv{};
+  if (warp == 0 && DC_INB(p, B, p.stride, 206)) mv = slot_load(p, base + B, lane);
+  uint32_t key = 0xFFFFFFFFu;
+  int slot = -1;
+  // (k, i) ranks below the best so far? Positions are read only to break ties.
+  auto take = [&](uint32_t k, int i) {
+    if (slot < 0 || k < key || (k == key && ps[i] > ps[slot])) {
+      key = k;
+      slot = i;
+    }
+  };
+  const float4* s4 = reinterpret_cast<const float4*>(p.score + base);  // the stride is a multiple of 128 slots
+  for (int e = tid; e < (n >> 2); e += kOneThreads) {
+    const float4 v = s4[e];
+    take(score_key(v.x), 4 * e);
+    take(score_key(v.y), 4 * e + 1);
+    take(score_key(v.z), 4 * e + 2);
+    take(score_key(v.w), 4 * e + 3);
+  }
+  for (int i = (n & ~3) + tid; i < n; i += kOneThreads) take(score_key(p.score[base + i]), i);
+  // the warp's lowest-ranked candidate: the lowest key (no valid key is
+  // 0xFFFFFFFF), among equal keys the latest position
+  auto reduce = [&] {
+    const uint32_t kmin = __reduce_min_sync(0xffffffffu, slot >= 0 ? key : 0xFFFFFFFFu);
+    unsigned who = __ballot_sync(0xffffffffu, slot >= 0 && key == kmin);
+    if (__popc(who) > 1) {
+      const bool in = who >> lane & 1u;
+      const int at = in ? ps[slot] : -1, pmax = __reduce_max_sync(0xffffffffu, at);
+      who = __ballot_sync(0xffffffffu, in && at == pmax);
+    }
+    key = kmin;
+    slot = who ? __shfl_sync(0xffffffffu, slot, __ffs(who) - 1) : -1;
+  };
+  reduce();
+  if (lane == 0) {
+    bkey[warp] = key;
+    bslot[warp] = slot;
+  }
+  __syncthreads();
+  if (warp > 0) return;
+  key = lane < kOneThreads / kWarp ? bkey[lane] : 0xFFFFFFFFu;
+  slot = lane < kOneThreads / kWarp ? bslot[lane] : -1;
+  reduce();
+  // slot B fills the evicted slot
+  if (slot >= 0 && slot < B) slot_store(p, base + slot, lane, mv);
+}
+
 // A row moves at most min(B, n - B) slots; with per-row budgets (B <= 0) at
 // most n / 2.
 static int max_moves(int n, int B) { return B > 0 ? (B < n - B ? B : n - B) : n / 2; }
 
-int evict_kernel_count(int n, int B) { return max_moves(n, B) > 0 ? 2 : 1; }
+static bool one_eviction(const Dev& p, int n, int B) { return !p.rowlen && B > 0 && n == B + 1; }
+
+int evict_kernel_count(const Dev& p, int n, int B) { return max_moves(n, B) > 0 && !one_eviction(p, n, B) ? 2 : 1; }
 
 void launch_evict(const Dev& p, int n, int B, cudaStream_t s) {
+  if (one_eviction(p, n, B)) {
+    evict_one_kernel<<<p.R, kOneThreads, 0, s>>>(p, n, B);
+    return;
+  }
   static bool attr = false;
   if (!attr) {
     if (cudaFuncSetAttribute(evict_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
