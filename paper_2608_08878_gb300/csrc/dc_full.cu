@@ -340,9 +340,14 @@ void full_t(const Dev& p, int n, int num_sms, const void* q, float* out, cudaStr
   la[0].id = cudaLaunchAttributeClusterDimension;
   cfg.attrs = la;
   cfg.numAttrs = 1;
-  static std::once_flag once;
-  static int active[kMaxSplits + 1];  // resident clusters of each size
-  std::call_once(once, [&] {
+  // resident clusters of each size, asked once per device
+  constexpr int kDevices = 64;
+  static std::once_flag once[kDevices];
+  static int active_on[kDevices][kMaxSplits + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) dev = 0;
+  int* const active = active_on[dev];
+  std::call_once(once[dev], [&] {
     const bool large = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     for (int k = 1; k <= kMaxSplits; ++k) {
       int m = 0;
