@@ -42,8 +42,10 @@
 // or both Z buffers, two tiles for one warpgroup could complete before it
 // waits for the first).
 //
-// TMEM columns: S tiles [0, 2 NQ), O [2 NQ, 2 NQ + 32) (rows in turn), logits
-// of heads 0..G-2 [2 NQ + 32, 256), policy layer [256, 512) (tiles in turn).
+// TMEM columns: S tiles [0, 2 NQ), O [2 NQ, 2 NQ + 64) (rows in turn; the even
+// and the odd tiles of a row have an accumulator each, summed in fp32 at the
+// end: the tensor core's accumulation loses a little at every tile), logits of
+// heads 0..G-2 [2 NQ + 64, 256), policy layer [256, 512) (tiles in turn).
 #pragma once
 #include "dc_fused_kernel.cuh"
 
@@ -56,12 +58,12 @@ constexpr int kBatchThreads = 128 + kBatchEpi;         // 16 warps: 128 register
 constexpr int kQSlots = 2;                             // query ring
 constexpr int kBatchRows = 24;                         // rows of a batch at most (their statistics' slots)
 
-// Tiles of a batch, whose logits wait on chip: heads 0..G-2 in TMEM (192
-// columns with G <= 4, 160 with G = 8), head G-1 in shared memory (512 B a
+// Tiles of a batch, whose logits wait on chip: heads 0..G-2 in TMEM (160
+// columns with G <= 4, 128 with G = 8), head G-1 in shared memory (512 B a
 // tile).
 template <int G>
 constexpr int batch_tiles() {
-  return G == 8 ? 22 : 48;
+  return G == 8 ? 18 : 48;
 }
 
 template <int G>
@@ -104,10 +106,13 @@ enum {
 // from the shared counter.
 __device__ __forceinline__ Item take_batch(const FusedStep& fs, const Dev& p, bool first) {
   const unsigned w = first ? blockIdx.x : gridDim.x + atomicAdd(fs.work + (fs.epoch & 1u), 1u);
-  const long long r0 = (long long)w * fs.batch_rows;
+  const bool full = w < (unsigned)fs.batch_full;
+  const int size = full ? fs.batch_rows : fs.batch_rest;
+  const long long r0 = full ? (long long)w * size
+                            : (long long)fs.batch_full * fs.batch_rows + (long long)(w - (unsigned)fs.batch_full) * size;
   if (r0 >= p.R) return Item{-1, 0, 0, 0};
   const int left = p.R - (int)r0;
-  return Item{(int)r0, left < fs.batch_rows ? left : fs.batch_rows, 0, -1};
+  return Item{(int)r0, left < size ? left : size, 0, -1};
 }
 
 // HEUR, GLOB, GRAPH as in fused_kernel: a heuristic scorer instead of the
@@ -119,7 +124,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
                  FusedStep fs, FusedPolicy fp) {
   constexpr int GS = G - 1;
   constexpr int NQ = q_rows<G>();
-  constexpr int kColO = 2 * NQ, kColStash = 2 * NQ + 32, kColZ = 256;
+  constexpr int kColO = 2 * NQ, kColStash = 2 * NQ + 64, kColZ = 256;
   static_assert(kColStash + GS * batch_tiles<G>() <= kColZ || GS == 0, "logits overlap the policy layer");
   static_assert(!GRAPH || (!HEUR && !GLOB), "device-counted steps: the plain step");
   if constexpr (GRAPH) {
@@ -402,8 +407,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
             const uint32_t plo = p_lo + (uint32_t)w * (4096 >> 4);
 #pragma unroll
             for (int ks = 0; ks < kTok / 16; ++ks)
-              mma_bf16_lo(tmem + kColO + 16 * ob, vlo + ks * (2048u >> 4), sdesc_hi(1024, 2), plo + ks * (512u >> 4),
-                          sdesc_hi(256, 6), id_pv, (j > 0 || ks > 0) ? 1u : 0u);
+              mma_bf16_lo(tmem + kColO + 32 * ob + 16 * (j & 1), vlo + ks * (2048u >> 4), sdesc_hi(1024, 2), plo + ks * (512u >> 4),
+                          sdesc_hi(256, 6), id_pv, (j > 1 || ks > 0) ? 1u : 0u);
             mma_commit(&bar[C_PEMPTY + w]);
             mma_commit(&bar[C_EMPTY + s]);
             if (j == nT - 1) {
@@ -887,8 +892,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
             ++ro;
             __syncwarp();
             tc_fence_after();
-            float o16[16];
-            tmem_ld16(lane_addr + kColO + 16 * ob, o16);
+            float o16[16], odd[16];
+            tmem_ld16(lane_addr + kColO + 32 * ob, o16);
+            tmem_ld16(lane_addr + kColO + 32 * ob + 16, odd);  // (not written when the row has one tile)
             tmem_ld_wait();
             tc_fence_before();
             __syncwarp();
@@ -897,7 +903,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
                                   (long long)(p.R / p.kvh) * p.qh * D, 115)) {
               float* op = fs.out + ((r / p.kvh) * p.qh + (r % p.kvh) * G) * D;
 #pragma unroll
-              for (int h = 0; h < G; ++h) op[h * D + tok] = o16[h] + o16[G + h];
+              for (int h = 0; h < G; ++h)
+                op[h * D + tok] = nT > 1 ? (o16[h] + odd[h]) + (o16[G + h] + odd[G + h]) : o16[h] + o16[G + h];
             }
             // ---------------- argtop_B and prune of the row: several evictions
             // here (radix select over its scores: every warp's are in), one by
@@ -944,7 +951,9 @@ static cudaError_t launch_batch_t(const FusedMaps& maps, const Dev& p, const Ste
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  const int items = (p.R + fs.batch_rows - 1) / fs.batch_rows, grid = items < num_sms ? items : num_sms;
+  const int rest = p.R - fs.batch_full * fs.batch_rows;
+  const int items = fs.batch_full + (fs.batch_rest ? (rest + fs.batch_rest - 1) / fs.batch_rest : 0);
+  const int grid = items < num_sms ? items : num_sms;
   if (!GRAPH)
     return launch_pdl(batch_kernel<D, G, HEUR, GLOB, GRAPH>, dim3(grid), dim3(kBatchThreads), kSmemBytes, s, maps.k,
                       maps.v, maps.k16, maps.v16, p, st, fs, fp);

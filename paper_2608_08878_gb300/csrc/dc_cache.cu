@@ -594,10 +594,15 @@ int effective_budget(const dc_cache* h, int budget, int n_cached, long long seen
   return (int)B;
 }
 
+// Whether a step over n tokens (after its append) is at most one token over
+// the budget that a call without one keeps: a steady step's schedule, the same
+// for dc_step and dc_decode_step.
+bool steady_step(const dc_cache* h, int n, long long seen) { return n - 1 <= effective_budget(h, 0, n, seen); }
+
 // Arguments of one fused launch; enables the half-row tail split when the
 // handle has exchange buffers and the step qualifies.
 dc::FusedStep fused_args(dc_cache* h, const dc::Step& st, const void* q, float* out, int do_evict, int B,
-                         int write_scores) {
+                         int write_scores, bool full = false) {
   dc::FusedStep fs{};
   fs.q = (const __nv_bfloat16*)q;
   fs.out = out;
@@ -610,8 +615,9 @@ dc::FusedStep fused_args(dc_cache* h, const dc::Step& st, const void* q, float* 
   fs.xflag = h->xflag;
   fs.xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
   fs.work = h->work;
-  fs.half_rows = (h->xflag && !h->per_row) ? dc::fused_half_rows(h->dev, st.n, fs, h->num_sms) : 0;
-  fs.batch_rows = dc::fused_batch_rows(h->dev, st.n, h->num_sms);
+  const bool steady = !full && steady_step(h, st.n, h->seen + 1);
+  fs.half_rows = (h->xflag && !h->per_row) ? dc::fused_half_rows(h->dev, st.n, fs, h->num_sms, steady) : 0;
+  if (!full && dc::fused_batches(h->dev, st.n, h->num_sms, steady)) dc::batch_items(h->dev, st.n, h->num_sms, &fs);
   // launch epoch: the queue counter is work[epoch & 1]; exchange flags hold
   // epoch * 4 + phase (1..3), so a flag left by an earlier launch never matches
   fs.epoch = ++h->epoch;
@@ -638,8 +644,8 @@ dc_status graph_step(dc_cache* h, const void* q, const void* k_new, const void* 
   fs.xflag = h->xflag;
   fs.xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
   fs.work = h->work;
-  fs.half_rows = h->xflag ? dc::fused_half_rows(h->dev, h->gstep.n, fs, h->num_sms) : 0;
-  fs.batch_rows = dc::fused_batch_rows(h->dev, h->gstep.n, h->num_sms);
+  fs.half_rows = h->xflag ? dc::fused_half_rows(h->dev, h->gstep.n, fs, h->num_sms, true) : 0;
+  if (dc::fused_batches(h->dev, h->gstep.n, h->num_sms, true)) dc::batch_items(h->dev, h->gstep.n, h->num_sms, &fs);
   fs.epoch = h->gepoch;
   cudaError_t e;
   {
@@ -651,14 +657,14 @@ dc_status graph_step(dc_cache* h, const void* q, const void* k_new, const void* 
 }
 
 // Whether a decode step over n tokens would split the fused grid's last wave.
-bool tail_split_applies(dc_cache* h, int n) {
+bool tail_split_applies(dc_cache* h, int n, bool steady) {
   if (!h->xflag) return false;
   dc::FusedStep fs{};
   fs.xstats = h->xstats;
   fs.xo = h->xo;
   fs.xsel = h->xsel;
   fs.xflag = h->xflag;
-  return dc::fused_half_rows(h->dev, n, fs, h->num_sms) > 0;
+  return dc::fused_half_rows(h->dev, n, fs, h->num_sms, steady) > 0;
 }
 
 }  // namespace
@@ -742,7 +748,7 @@ dc_status dc_step(dc_cache* h, const void* q, const void* k_new, const void* v_n
     return dc_evict(h, budget);
   }
   const int B = effective_budget(h, budget, n1, h->seen + 1);
-  if (!h->per_row && B < n1 - 1 && (tail_split_applies(h, n1) || n1 - B > kFusedEvictMax)) {
+  if (!h->per_row && B < n1 - 1 && (tail_split_applies(h, n1, steady_step(h, n1, h->seen + 1)) || n1 - B > kFusedEvictMax)) {
     // several evictions need the whole row's scores in one CTA: with half
     // rows this step runs as the decode kernel plus the eviction kernel; so
     // does a step with many evictions (a prompt compression), whose moves the
@@ -893,7 +899,7 @@ dc_status dc_step_host_async(dc_cache* h, const void* q, const void* k_new, cons
 dc_status dc_engine(dc_cache* h, int n, int* engine) {
   if (!valid(h) || !engine) return DC_ERR_INVALID_ARG;
   const int nn = n > 0 ? n : h->n + 1;
-  *engine = !use_fused(h, nn) ? 1 : dc::fused_batch_rows(h->dev, nn, h->num_sms) ? 3 : 2;
+  *engine = !use_fused(h, nn) ? 1 : dc::fused_pairs(h->dev, nn, h->num_sms) ? 3 : 2;
   return DC_OK;
 }
 
@@ -960,7 +966,7 @@ dc_status dc_full_decode(dc_cache* h, const void* q, float* out) {
     // the fused kernel's attention-only variant (TMA + tensor cores)
     dc::Step st{};
     st.n = h->n;
-    const dc::FusedStep fs = fused_args(h, st, q, out, 0, 0, 0);
+    const dc::FusedStep fs = fused_args(h, st, q, out, 0, 0, 0, true);
     cudaError_t e;
     {
       Phase ph(h, DC_PHASE_FULL, 1);

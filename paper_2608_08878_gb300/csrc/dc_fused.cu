@@ -1,7 +1,7 @@
 // dc_fused.cu -- the fused engine's host side and its main instantiations
 // (per-row selection with the policy MLP; rows within and past the on-chip
 // logit capacity). The kernel itself is in dc_fused_kernel.cuh.
-#include "dc_fused_kernel.cuh"
+#include "dc_batch_kernel.cuh"
 
 namespace dc {
 
@@ -17,24 +17,58 @@ bool fused_eligible(const Dev& p, int n) {
 
 int fused_smem_bytes() { return Smem<4>::BYTES; }
 
-int fused_batch_rows(const Dev& p, int n, int num_sms) {
+static int batch_tiles_of(int G) { return G == 8 ? batch_tiles<8>() : batch_tiles<4>(); }
+
+void batch_items(const Dev& p, int n, int num_sms, FusedStep* fs) {
+  const int nT = (n + kTok - 1) / kTok, fit = batch_tiles_of(p.G) / nT, cap = fit < kBatchRows ? fit : kBatchRows;
+  // as many rounds of full batches as all SMs can take, then one round of the
+  // smallest batches that hold the rest: every SM gets the same number of rows,
+  // to within one
+  const int rounds = p.R / (num_sms * cap), rest = p.R - rounds * num_sms * cap;
+  fs->batch_rows = cap;
+  fs->batch_full = rounds * num_sms;
+  fs->batch_rest = (rest + num_sms - 1) / num_sms;
+}
+
+// Row pairs (one row per warpgroup, two per CTA), as they were chosen before
+// batches took their place: short rows (at most 21 tiles), more rows than SMs,
+// an even row count, the plain step (policy scorer, equal lengths, per-row
+// selection), and the cheaper critical path of a CTA in tokens of streaming
+// time: a row costs its n tokens plus ~350 of serial epilogue, a pair 2n plus
+// ~410.
+bool fused_pairs(const Dev& p, int n, int num_sms) {
   const int nT = (n + kTok - 1) / kTok;
   if (!(p.seq_rows == 0 && p.rowlen == nullptr && p.scorer == 0 && p.G <= 4 && p.R % 2 == 0 && p.R > num_sms &&
         nT >= 1 && nT <= 21))
-    return 0;
-  // Critical path of a CTA in units of one token's streaming time at an SM's
-  // share of the bandwidth (measured with per-row timestamps): a row costs its
-  // n tokens plus ~350 of serial epilogue (statistics merge, output, select), a
-  // pair 2n plus ~410. Pairs halve the serial part per row but make the last
-  // wave coarser: the cheaper schedule wins.
+    return false;
   const int rem = p.R % num_sms;
   const double waves1 = p.R / num_sms + (rem == 0 ? 0.0 : 2 * rem <= num_sms ? 0.5 : 1.0);
   const double waves2 = (p.R / 2 + num_sms - 1) / num_sms;
-  return waves2 * (2.0 * n + 410.0) < waves1 * (n + 350.0) ? batch_rows_per_item(p, n, num_sms) : 0;
+  return waves2 * (2.0 * n + 410.0) < waves1 * (n + 350.0);
 }
 
-int fused_half_rows(const Dev& p, int n, const FusedStep& fs, int num_sms) {
-  if (fused_batch_rows(p, n, num_sms)) return 0;
+bool fused_batches(const Dev& p, int n, int num_sms, bool steady) {
+  // Rows of equal length whose logits fit on chip (6144 tokens, 2304 with eight
+  // query heads). Batches measured faster than whole rows at every such size
+  // (us a step, whole -> batches: 160 rows x 411 27.5 -> 17.1, 512 x 1025 72.5 ->
+  // 52.8, 256 x 2689 66.4 -> 59.7, 1024 x 4097 350 -> 342; GQA-8 512 x 411 59.4 ->
+  // 32.4; H2O 512 x 411 49.0 -> 26.1; 112 x 2049 27.5 -> 25.3, 8 x 129 11.0 -> 9.9;
+  // equal within 3% at one query head of 64 dims), and than halves below 30
+  // tiles (72 x 2049 37.0 -> 24.5; 8 x 4097: 32.8 in halves, 38.9 in batches).
+  //
+  // A row's statistics come from one warpgroup here and from two, merged in
+  // another order, on whole rows: their last bits differ. So steps that may
+  // evict many tokens, whose selection cuts through near-ties, keep the schedule
+  // that the row-pair rule (the first to put rows on one warpgroup) gives them;
+  // steady steps take the faster one.
+  const int nT = (n + kTok - 1) / kTok;
+  if (p.rowlen || nT > batch_tiles_of(p.G)) return false;
+  if (fused_pairs(p, n, num_sms)) return true;
+  return steady && !(4 * p.R <= num_sms && nT >= 30);
+}
+
+int fused_half_rows(const Dev& p, int n, const FusedStep& fs, int num_sms, bool steady) {
+  if (fused_batches(p, n, num_sms, steady)) return 0;
   const int grid = p.R < num_sms ? p.R : num_sms, rem = p.R % grid;
   const int nT = (n + kTok - 1) / kTok;
   const bool ok = fs.xflag && fs.xstats && fs.xo && fs.xsel && nT >= 2 && (!fs.do_evict || fs.B >= n || fs.B == n - 1);
@@ -50,9 +84,9 @@ int fused_half_rows(const Dev& p, int n, const FusedStep& fs, int num_sms) {
 cudaError_t launch_fused_step(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                               const FusedPolicy& fp, int num_sms, cudaStream_t s) {
   // the other variants are instantiated in their own translation units
+  if (fs.batch_rows) return launch_fused_batch(maps, p, st, fs, fp, num_sms, s);
   if (p.seq_rows) return launch_fused_glob(maps, p, st, fs, fp, num_sms, s);
   if (p.rowlen || p.scorer != 0) return launch_fused_heur_perrow(maps, p, st, fs, fp, num_sms, s);
-  if (fs.batch_rows) return launch_fused_batch(maps, p, st, fs, fp, num_sms, s);
   const int grid = fused_grid(p, fs, num_sms);
   const bool lg = st.n > fused_onchip_tokens(p.G);
 #define DC_FUSED_LAUNCH(D, G) \

@@ -40,7 +40,9 @@ struct FusedStep {
   int* xsel;         // [half_rows][2][4]
   unsigned* xflag;   // [half_rows][2]
   int xslots;        // exchange slots allocated (bounds of the four above)
-  int batch_rows;    // rows per work item when the step runs on batches of rows (batch_kernel), else 0
+  // batches of rows (batch_kernel): the first batch_full work items hold
+  // batch_rows rows each, the others batch_rest; batch_rows 0: not on batches
+  int batch_rows, batch_full, batch_rest;
 };
 
 // Exchange buffer sizes (floats / ints) for a grid of `grid` CTAs.
@@ -80,20 +82,19 @@ cudaError_t make_fused_maps(const Dev& p, FusedMaps* maps, const char** why);
 // FusedPolicy fields and the host copy of the weight tile (128 * 32 bf16).
 void prepare_policy(const float* blob, int H, int layernorm, FusedPolicy* fp, std::vector<__nv_bfloat16>* wtile);
 
-// Rows per work item when a step over n tokens runs on batches of rows (each
-// warpgroup of a CTA on rows of its own, dc_batch_kernel.cuh), 0 when it does
-// not: short rows, more rows than SMs, an even row count, the plain step
-// (policy scorer, equal lengths, per-row selection).
-int fused_batch_rows(const Dev& p, int n, int num_sms);
-// Tiles of a row that fit the batch schedule, and the rows per item there.
-int batch_row_tiles(int G);
-int batch_rows_per_item(const Dev& p, int n, int num_sms);
+// Whether a step over n tokens runs on batches of rows (dc_batch_kernel.cuh).
+// `steady`: every row is at most one token over its budget. fused_pairs is the
+// part of the rule that dc_engine reports.
+bool fused_pairs(const Dev& p, int n, int num_sms);
+bool fused_batches(const Dev& p, int n, int num_sms, bool steady);
+// The division of the rows into work items there: see FusedStep.
+void batch_items(const Dev& p, int n, int num_sms, FusedStep* fs);
 
 // How many rows a step over n tokens splits into halves (see FusedStep): every
 // row when rows are at most half the SMs and at least 12 tiles long, else the
 // remainder of R over the grid when it is at most half the grid, else 0 (and 0
 // on batches of rows).
-int fused_half_rows(const Dev& p, int n, const FusedStep& fs, int num_sms);
+int fused_half_rows(const Dev& p, int n, const FusedStep& fs, int num_sms, bool steady);
 
 cudaError_t launch_fused_step(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                               const FusedPolicy& fp, int num_sms, cudaStream_t s);
@@ -105,6 +106,10 @@ cudaError_t launch_fused_heur_perrow(const FusedMaps& maps, const Dev& p, const 
                                      const FusedPolicy& fp, int num_sms, cudaStream_t s);
 cudaError_t launch_fused_glob(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                               const FusedPolicy& fp, int num_sms, cudaStream_t s);
+// The heuristic scorers and the global token mode on batches of rows
+// (dc_batch_modes.cu).
+cudaError_t launch_batch_modes(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
+                               const FusedPolicy& fp, int num_sms, cudaStream_t s);
 // Batches of rows (dc_batch.cu), FusedStep::batch_rows > 0.
 cudaError_t launch_fused_batch(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                               const FusedPolicy& fp, int num_sms, cudaStream_t s);
