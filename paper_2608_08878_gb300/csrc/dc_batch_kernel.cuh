@@ -19,13 +19,17 @@
 // more than it gave (1380 us).
 //
 // A row's arithmetic and its order do not depend on the batch or on the tiles'
-// assignment: the statistics of a row come from one warpgroup in tile order,
-// and the V pass works token by token.
+// assignment: the statistics of a row come from one warpgroup in tile order
+// (in the order of the schedule that the step had before, so that scores, and
+// with them the tokens kept, are bit for bit what they were: one query head's
+// softmax sum off by its last bit changed the token evicted in one row-step of
+// 6000 to 25000), and the V pass works token by token.
 //
 // Warp roles (512 threads, 128 registers each):
 //   warp 0      producer: takes items, loads each row's current, previous and
-//               departing queries and their statistics a row ahead of its
-//               tiles, streams K then V tiles (TMA);
+//               departing queries and their statistics (and its new pair, which
+//               it appends) a row ahead of its tiles, streams K then V tiles
+//               (TMA);
 //   warp 1      MMA issuer (S = K Q^T, O^T += V^T P^T);
 //   warp 2      policy-layer MMA issuer (Z = A W^T);
 //   warp 3      mover: the one-eviction select of every row and its move;
@@ -78,8 +82,8 @@ struct BatchSmem {
   static constexpr int SC = AUX + kStages * kAuxBytes;
   static constexpr int QST = SC + batch_tiles<G>() * kTok * 4;       // window queries' statistics: [slots][6][G] floats
   static constexpr int RST = QST + kQSlots * 6 * G * 4;              // rows' final statistics: [kBatchRows][3][G]
-  static constexpr int RED = RST + kBatchRows * 3 * G * 4;           // merge scratch: [2 (row in turn)][warps][G][3]
-  static constexpr int CAND = RED + 2 * 4 * kBatchWg * G * 3 * 4;    // [kBatchRows][warps][4]: key, slot, position
+  static constexpr int RED = RST + kBatchRows * 3 * G * 4;           // merge scratch: [2 (row in turn)][warps x 2][G][3]
+  static constexpr int CAND = RED + 2 * 8 * kBatchWg * G * 3 * 4;    // [kBatchRows][warps][4]: key, slot, position
   static constexpr int SEL = CAND + kBatchRows * 4 * kBatchWg * 16;   // select scratch per warpgroup: 288 ints
   static constexpr int MISC = (SEL + kBatchWg * 288 * 4 + 15) / 16 * 16;
   static constexpr int BYTES = MISC + 1024 + 1024;                   // misc area + alignment slack
@@ -211,6 +215,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     prefetch_tmap(&tmV16);
   }
   grid_dep_wait();
+  // the launch after this one may start its set-up (where an SM has room, at the
+  // latest when a CTA leaves), one launch ahead at most
+  if constexpr (!GRAPH) grid_dep_launch();
   // the next launch's queue counter (this launch uses the other one)
   if (blockIdx.x == 0 && threadIdx.x == 0) fs.work[(fs.epoch + 1u) & 1u] = 0u;
   __syncthreads();
@@ -224,8 +231,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     const uint64_t pol = l2_evict_first_policy();
     constexpr int QCH = G * (D / 8);                 // 16-byte chunks of a row's G query heads
     constexpr int QIT = (QCH + kWarp - 1) / kWarp;   // per lane
-    uint4 qcur[QIT], qprev[QIT], qdep[QIT];
+    uint4 qcur[QIT], qprev[QIT], qdep[QIT], kvn = make_uint4(0, 0, 0, 0);
     float4 rstat;
+    constexpr int VPR = D / 8;  // 16-byte chunks of a K (or V) row
     const int sh = lane % G, sdep = lane / G;        // window statistics: lanes [0, 2G), head and query
     auto q_ok = [&](int rq) {
       return DC_INB(p, (long long)((rq / p.kvh) * p.qh + (rq % p.kvh) * G) * D + G * D - 1,
@@ -246,6 +254,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         qprev[u] = ld && st.has_prev ? prev[e] : make_uint4(0, 0, 0, 0);
         qdep[u] = ld && st.has_dep ? dep[e] : make_uint4(0, 0, 0, 0);
       }
+      if (fs.k_new && lane < 2 * VPR)
+        kvn = (lane < VPR ? fs.k_new : fs.v_new)[(size_t)rq * VPR + lane % VPR];
       rstat = make_float4(0.f, 0.f, 0.f, 0.f);
       if (lane < 2 * G && ok)
         rstat = reinterpret_cast<const float4*>(p.ring_stats)[((size_t)rq * p.w + (sdep ? st.slot : st.slot_prev)) * G + sh];
@@ -273,6 +283,29 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         w[G + sh] = rstat.w;
         w[2 * G + sh] = rstat.z;
       }
+      if (fs.k_new && DC_INB(p, n - 1, p.cap, 301) && DC_INB(p, rq, p.R, 301)) {
+        // the new pair into slot n - 1, with |v| and a clean state (as the append
+        // kernel does it)
+        const size_t at = (size_t)rq * p.stride + (n - 1);
+        if (lane < VPR) reinterpret_cast<uint4*>(p.K)[at * VPR + lane] = kvn;
+        else if (lane < 2 * VPR) reinterpret_cast<uint4*>(p.V)[at * VPR + lane - VPR] = kvn;
+        const uint32_t w4[4] = {kvn.x, kvn.y, kvn.z, kvn.w};
+        float ss = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float x0 = bf16lo(w4[e]), x1 = bf16hi(w4[e]);
+          ss = fmaf(x0, x0, ss);
+          ss = fmaf(x1, x1, ss);
+        }
+#pragma unroll
+        for (int off = 1; off < VPR; off <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+        if (lane == VPR) {
+          p.pos[at] = st.p_newest;
+          p.vnorm[at] = sqrtf(ss);
+          p.SZ[at] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (p.acc) p.acc[at] = 0.f;
+        }
+      }
       fence_proxy_async();
       __syncwarp();
     };
@@ -287,11 +320,11 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
       return v;
     };
     int g = 0, issued = 0, rs = 0;
-    // one lane: the K or V tiles of row rt into the stage ring; false: winding down
-    auto issue = [&](int rt, bool vpass) {
+    // one lane: K or V tiles [j0, j1) of row rt into the stage ring; false: winding down
+    auto issue = [&](int rt, bool vpass, int j0, int j1) {
       const CUtensorMap* tm = vpass ? &tmV : &tmK;
       const CUtensorMap* tm16 = vpass ? &tmV16 : &tmK16;
-      for (int j = 0; j < nT; ++j, ++g) {
+      for (int j = j0; j < j1; ++j, ++g) {
         const int s = g % kStages;
         if (!mbar_wait(&bar[C_EMPTY + s], ((g / kStages) & 1) ^ 1, abort, p.dbg, 2u, (unsigned)g)) return false;
         const int valid = n - j * kTok < kTok ? n - j * kTok : kTok;
@@ -339,14 +372,23 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         store_q(it.x + i, slot);
         if (lane == 0) mbar_arrive(&bar[C_QFULL + slot]);
         if (i + 1 < it.y) load_q(it.x + i + 1);
-        if (elect_one()) ok = issue(it.x + i, false);
+        // the last tile holds the new pair: its copies come after the writes of
+        // it, whose latency the tiles before cover
+        if (fs.k_new) {
+          if (elect_one()) ok = issue(it.x + i, false, 0, nT - 1);
+          fence_proxy_async_global();
+          __syncwarp();
+          if (elect_one()) ok = ok && issue(it.x + i, false, nT - 1, nT);
+        } else if (elect_one()) {
+          ok = issue(it.x + i, false, 0, nT);
+        }
         ok = __all_sync(0xffffffffu, ok);
       }
       if (!ok) break;
       const int2 nx = take(false);
       if (nx.x >= 0) load_q(nx.x);
       if (elect_one())
-        for (int i = 0; i < it.y && ok; ++i) ok = issue(it.x + i, true);
+        for (int i = 0; i < it.y && ok; ++i) ok = issue(it.x + i, true, 0, nT);
       ok = __all_sync(0xffffffffu, ok);
       it = nx;
     }
@@ -545,9 +587,15 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         const int rs = rs0 + i, slot = rs % kQSlots;
         const float* wq = qst + slot * 6 * G;
         const size_t rbase = (size_t)r * stride;
-        float m[G], l[G], u[G];
+        // online softmax state; with batch_dual, even and odd tiles apart, as on
+        // whole rows, where each of two warpgroups takes every other tile
+        float m[G], l[G], u[G], m2[G], l2[G], u2[G];
 #pragma unroll
-        for (int h = 0; h < G; ++h) { m[h] = kNoMax; l[h] = 0.f; u[h] = 0.f; }
+        for (int h = 0; h < G; ++h) {
+          m[h] = m2[h] = kNoMax;
+          l[h] = l2[h] = 0.f;
+          u[h] = u2[h] = 0.f;
+        }
         for (int j = 0; j < nT; ++j) {
           const int gj = g + i * nT + j, s = gj % kStages, b = (gs + i * nT + j) & 1;
           mbar_wait(&bar[C_SFULL + 2 * wg + b], (sph >> b) & 1, abort, p.dbg, 6u, (unsigned)gj);
@@ -572,7 +620,10 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
           const int ti = j * kTok + tok, lt = i * nT + j;
           if (ti < n) {
 #pragma unroll
-            for (int h = 0; h < G; ++h) online_add(m[h], l[h], u[h], S16[h], c);
+            for (int h = 0; h < G; ++h) {
+              if (fs.batch_dual && (j & 1)) online_add(m2[h], l2[h], u2[h], S16[h], c);
+              else online_add(m[h], l[h], u[h], S16[h], c);
+            }
             if (!GLOB && (st.has_prev || st.has_dep)) {
               // terms of the previous and the departing query, masked (x 1 or x 0,
               // both exact) where the token was not yet in the cache at that step
@@ -593,47 +644,65 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         if (lane == 0) mbar_arrive(&bar[C_QEMPTY + slot]);
         // ---------------- row softmax statistics (deterministic merge order):
         // the maximum first, then every partial (l, u) rescaled to it and summed
-        float* redp = red + ((i / kBatchWg) & 1) * 4 * kBatchWg * G * 3 + wg * 4 * G * 3;
+        float* redp = red + ((i / kBatchWg) & 1) * 8 * kBatchWg * G * 3 + wg * 8 * G * 3;
+        // (every operation rounded as written: a contracted first addition
+        // would change the sums' last bits from one instantiation to another)
+        auto partial = [&](const float (&pm)[G], const float (&pl)[G], const float (&pu)[G], int at) {
 #pragma unroll
-        for (int h = 0; h < G; ++h) {
-          float mm = m[h];
+          for (int h = 0; h < G; ++h) {
+            float mm = pm[h];
 #pragma unroll
-          for (int off = 16; off > 0; off >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, off));
-          // (every operation rounded as written: a contracted first addition
-          // would change the sums' last bits from one instantiation to another)
-          const float dm = __fmul_rn(__fsub_rn(m[h], mm), c), f = ex2(dm);
-          float ll = __fmul_rn(l[h], f), uu = __fmul_rn(__fmaf_rn(l[h], dm, u[h]), f);
+            for (int off = 16; off > 0; off >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, off));
+            const float dm = __fmul_rn(__fsub_rn(pm[h], mm), c), f = ex2(dm);
+            float ll = __fmul_rn(pl[h], f), uu = __fmul_rn(__fmaf_rn(pl[h], dm, pu[h]), f);
 #pragma unroll
-          for (int off = 16; off > 0; off >>= 1) {
-            ll = __fadd_rn(ll, __shfl_xor_sync(0xffffffffu, ll, off));
-            uu = __fadd_rn(uu, __shfl_xor_sync(0xffffffffu, uu, off));
+            for (int off = 16; off > 0; off >>= 1) {
+              ll = __fadd_rn(ll, __shfl_xor_sync(0xffffffffu, ll, off));
+              uu = __fadd_rn(uu, __shfl_xor_sync(0xffffffffu, uu, off));
+            }
+            if (lane == 0) {
+              float* rw = redp + (at * G + h) * 3;
+              rw[0] = mm;
+              rw[1] = ll;
+              rw[2] = uu;
+            }
           }
-          if (lane == 0) {  // (merged in the order of token quarters 2, 3, 0, 1)
-            float* rw = redp + ((quad ^ 2) * G + h) * 3;
-            rw[0] = mm;
-            rw[1] = ll;
-            rw[2] = uu;
-          }
-        }
+        };
+        // merged in the order of token quarters 2, 3, 0, 1; with batch_dual the
+        // tiles of whole rows' warpgroup 0 first: the even ones, or on every
+        // other item of a CTA with an odd tile count the odd ones
+        const int flip = fs.batch_dual ? ((r / fs.batch_sms) * nT) & 1 : 0;
+        partial(m, l, u, 4 * flip + (quad ^ 2));
+        if (fs.batch_dual) partial(m2, l2, u2, 4 * (flip ^ 1) + (quad ^ 2));
         sync();  // (the scratch alternates between the warpgroup's rows: one barrier per row)
         // one lane per head merges the warps' partials, publishes the row's
         // statistics and pushes (m, l, H, -log2 l) into the ring slot of this
         // step (the query loader wrote the query there)
         if (tid < G) {
-          const int h = tid;
+          const int h = tid, parts = fs.batch_dual ? 8 : 4;
           float mm = kNoMax;
 #pragma unroll
-          for (int w = 0; w < 4; ++w) mm = fmaxf(mm, redp[(w * G + h) * 3 + 0]);
+          for (int w = 0; w < 8; ++w)
+            if (w < parts) mm = fmaxf(mm, redp[(w * G + h) * 3 + 0]);
           float ll = 0.f, uu = 0.f;
 #pragma unroll
-          for (int w = 0; w < 4; ++w) {
+          for (int w = 0; w < 8; ++w) {
+            if (w >= parts) break;
             const float lw = redp[(w * G + h) * 3 + 1];
             const float dm = __fmul_rn(__fsub_rn(redp[(w * G + h) * 3 + 0], mm), c), f = ex2(dm);
             ll = __fmaf_rn(lw, f, ll);
             uu = __fmaf_rn(__fmaf_rn(lw, dm, redp[(w * G + h) * 3 + 2]), f, uu);
           }
           // H = ln l - ln 2 u / l
-          const float nl = -log2f(ll), hh = logf(ll) - 0.69314718055994531f * (uu / ll);
+          float nl, hh;
+          if (fs.batch_dual) {  // as whole rows do, from the hardware log2 and divide (l >= 1)
+            const float lg = lg2_approx(ll);
+            nl = -lg;
+            hh = 0.69314718055994531f * (lg - __fdividef(uu, ll));
+          } else {
+            nl = -log2f(ll);
+            hh = logf(ll) - 0.69314718055994531f * (uu / ll);
+          }
           rst[(i * 3 + 0) * G + h] = mm;
           rst[(i * 3 + 1) * G + h] = nl;
           rst[(i * 3 + 2) * G + h] = hh;

@@ -624,12 +624,21 @@ dc::FusedStep fused_args(dc_cache* h, const dc::Step& st, const void* q, float* 
   return fs;
 }
 
+// Whether the next decode step, over n tokens, appends its new pairs in the
+// step's own kernel.
+bool kernel_appends(const dc_cache* h, int n) {
+  return !h->per_row && use_fused(h, n) && dc::batch_appends(h->dev, h->num_sms) &&
+         dc::fused_batches(h->dev, n, h->num_sms, steady_step(h, n, h->seen + 1));
+}
+
 // One device-counted step (graph mode): the append and the fused step with the
 // base arguments, which the kernels advance by the device's step count; the
 // host's mirror of the step state stays at the base until the mode ends.
 dc_status graph_step(dc_cache* h, const void* q, const void* k_new, const void* v_new, float* out, int budget) {
   if (budget > 0 && budget != h->budget) return fail(h, DC_ERR_INVALID_ARG, "graph mode keeps the configured budget");
-  {
+  const bool batches = dc::fused_batches(h->dev, h->gstep.n, h->num_sms, true);
+  const bool appends = batches && dc::batch_appends(h->dev, h->num_sms);
+  if (!appends) {
     Phase ph(h, DC_PHASE_APPEND, 1);
     dc::launch_append(h->dev, k_new, v_new, 1, h->n, h->gstep.p_newest, h->stream);
   }
@@ -645,7 +654,11 @@ dc_status graph_step(dc_cache* h, const void* q, const void* k_new, const void* 
   fs.xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
   fs.work = h->work;
   fs.half_rows = h->xflag ? dc::fused_half_rows(h->dev, h->gstep.n, fs, h->num_sms, true) : 0;
-  if (dc::fused_batches(h->dev, h->gstep.n, h->num_sms, true)) dc::batch_items(h->dev, h->gstep.n, h->num_sms, &fs);
+  if (batches) dc::batch_items(h->dev, h->gstep.n, h->num_sms, &fs);
+  if (appends) {
+    fs.k_new = (const uint4*)k_new;
+    fs.v_new = (const uint4*)v_new;
+  }
   fs.epoch = h->gepoch;
   cudaError_t e;
   {
@@ -677,14 +690,19 @@ dc_status dc_decode_step(dc_cache* h, const void* q, const void* k_new, const vo
     return fail(h, DC_ERR_INVALID_ARG, "q, k_new and v_new must be 16-byte aligned");
   if (h->n + 1 > h->capacity) return fail(h, DC_ERR_CAPACITY, "decode step exceeds capacity");
   if (h->seen + 1 > 0x7FFFFFFFll) return fail(h, DC_ERR_CAPACITY, "position counter overflow");
-  {
+  const bool appends = kernel_appends(h, h->n + 1);
+  if (!appends) {
     Phase ph(h, DC_PHASE_APPEND, h->per_row ? 2 : 1);
     dc::launch_append(h->dev, k_new, v_new, 1, h->n, (int)h->seen, h->stream);
     if (h->per_row) dc::launch_rowlen_add(h->dev, 1, h->stream);
   }
   const dc::Step st = begin_step(h);
   if (use_fused(h, st.n)) {
-    const dc::FusedStep fs = fused_args(h, st, q, out, 0, 0, h->dev.seq_rows ? 0 : 1);
+    dc::FusedStep fs = fused_args(h, st, q, out, 0, 0, h->dev.seq_rows ? 0 : 1);
+    if (appends) {
+      fs.k_new = (const uint4*)k_new;
+      fs.v_new = (const uint4*)v_new;
+    }
     cudaError_t e;
     {
       Phase ph(h, DC_PHASE_ATTEND, 1);
@@ -759,7 +777,8 @@ dc_status dc_step(dc_cache* h, const void* q, const void* k_new, const void* v_n
     return dc_evict(h, budget);
   }
   if (h->seen + 1 > 0x7FFFFFFFll) return fail(h, DC_ERR_CAPACITY, "position counter overflow");
-  {
+  const bool appends = kernel_appends(h, n1);
+  if (!appends) {
     Phase ph(h, DC_PHASE_APPEND, h->per_row ? 2 : 1);
     dc::launch_append(h->dev, k_new, v_new, 1, h->n, (int)h->seen, h->stream);
     if (h->per_row) dc::launch_rowlen_add(h->dev, 1, h->stream);
@@ -789,7 +808,11 @@ dc_status dc_step(dc_cache* h, const void* q, const void* k_new, const void* v_n
     return DC_OK;
   }
   const int keep = std::min(st.n, B);
-  const dc::FusedStep fs = fused_args(h, st, q, out, keep < st.n ? 1 : 0, keep, 0);
+  dc::FusedStep fs = fused_args(h, st, q, out, keep < st.n ? 1 : 0, keep, 0);
+  if (appends) {
+    fs.k_new = (const uint4*)k_new;
+    fs.v_new = (const uint4*)v_new;
+  }
   cudaError_t e;
   {
     Phase ph(h, DC_PHASE_ATTEND, 1);

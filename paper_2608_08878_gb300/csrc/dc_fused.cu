@@ -28,6 +28,20 @@ void batch_items(const Dev& p, int n, int num_sms, FusedStep* fs) {
   fs->batch_rows = cap;
   fs->batch_full = rounds * num_sms;
   fs->batch_rest = (rest + num_sms - 1) / num_sms;
+  // (a few rows, or rows that ran in halves before: no whole-row order to keep)
+  fs->batch_dual = p.R > 16 && !fused_pairs(p, n, num_sms) && !(2 * p.R <= num_sms && nT >= 12);
+  fs->batch_sms = num_sms;
+}
+
+bool batch_appends(const Dev& p, int num_sms) {
+  // The append kernel and the gap after it cost a step 1 to 2.5 us; in the step's
+  // kernel the producer writes each row's new pair ahead of its last tile. That
+  // gains while a CTA has few rows (us a step, append kernel -> in the kernel:
+  // 8 rows x 129 10.4 -> 8.8, 152 x 411 16.4 -> 13.6, 256 x 411 19.2 -> 18.3, 1024 x
+  // 411 49.6 -> 47.3, 1024 x 4097 345.7 -> 342.5) and costs the producer more
+  // than it gains with many (4096 x 411 166.6 -> 168.4, 16384 x 411 638 -> 660).
+  // The global mode's append also clears the sequence's ring.
+  return p.seq_rows == 0 && p.R <= 16 * num_sms;
 }
 
 // Row pairs (one row per warpgroup, two per CTA), as they were chosen before
@@ -56,11 +70,11 @@ bool fused_batches(const Dev& p, int n, int num_sms, bool steady) {
   // equal within 3% at one query head of 64 dims), and than halves below 30
   // tiles (72 x 2049 37.0 -> 24.5; 8 x 4097: 32.8 in halves, 38.9 in batches).
   //
-  // A row's statistics come from one warpgroup here and from two, merged in
-  // another order, on whole rows: their last bits differ. So steps that may
-  // evict many tokens, whose selection cuts through near-ties, keep the schedule
-  // that the row-pair rule (the first to put rows on one warpgroup) gives them;
-  // steady steps take the faster one.
+  // A row's statistics come out here bit for bit as on the schedule that ran the
+  // row before (whole rows, or row pairs: FusedStep::batch_dual), but not as in
+  // halves, whose last bits differ. So steps that may evict many tokens, whose
+  // selection cuts through near-ties, keep the schedule that they had; steady
+  // steps take the faster one.
   const int nT = (n + kTok - 1) / kTok;
   if (p.rowlen || nT > batch_tiles_of(p.G)) return false;
   if (fused_pairs(p, n, num_sms)) return true;

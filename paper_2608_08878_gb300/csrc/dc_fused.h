@@ -24,6 +24,10 @@ struct FusedMaps {
 struct FusedStep {
   const __nv_bfloat16* q;
   float* out;
+  // batches of rows: the step's new pairs, which the kernel appends itself; null
+  // when the append kernel has run
+  const uint4* k_new;
+  const uint4* v_new;
   int do_evict;      // 1: select and compact in the same kernel
   int B;             // tokens to keep when do_evict
   int write_scores;  // 1: also store scores in Dev::score (for dc_evict)
@@ -43,6 +47,8 @@ struct FusedStep {
   // batches of rows (batch_kernel): the first batch_full work items hold
   // batch_rows rows each, the others batch_rest; batch_rows 0: not on batches
   int batch_rows, batch_full, batch_rest;
+  int batch_sms;     // SMs (the whole-row schedule's CTAs)
+  int batch_dual;    // 1: rows' statistics in the order of whole rows (see batch_kernel), 0: of row pairs
 };
 
 // Exchange buffer sizes (floats / ints) for a grid of `grid` CTAs.
@@ -89,6 +95,8 @@ bool fused_pairs(const Dev& p, int n, int num_sms);
 bool fused_batches(const Dev& p, int n, int num_sms, bool steady);
 // The division of the rows into work items there: see FusedStep.
 void batch_items(const Dev& p, int n, int num_sms, FusedStep* fs);
+// Whether such a step appends its new pairs in the kernel.
+bool batch_appends(const Dev& p, int num_sms);
 
 // How many rows a step over n tokens splits into halves (see FusedStep): every
 // row when rows are at most half the SMs and at least 12 tiles long, else the
