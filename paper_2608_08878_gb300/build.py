@@ -30,7 +30,7 @@ BUILD_DEBUG = os.path.join(HERE, "_build_debug")
 
 MAIN_SOURCES = ["dc_cache.cu", "dc_split.cu", "dc_evict.cu", "dc_full.cu", "dc_fused.cu", "dc_noalloc.cu",
                 "dc_train.cu", "dc_global.cu", "dc_fused_modes.cu", "dc_fused_glob.cu",
-                "dc_batch.cu", "dc_batch_modes.cu", "dc_selftest.cu", "dc_fused_graph.cu"]
+                "dc_batch.cu", "dc_batch_modes.cu", "dc_batch_cluster.cu", "dc_selftest.cu", "dc_fused_graph.cu"]
 SYNTH_SOURCES = ["synth.cu"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -23,6 +23,7 @@ static cudaError_t launch_plain(const FusedMaps& maps, const Dev& p, const Step&
 
 cudaError_t launch_fused_batch(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                                const FusedPolicy& fp, int num_sms, cudaStream_t s) {
+  if (fs.batch_cluster > 1) return launch_batch_cluster(maps, p, st, fs, fp, num_sms, false, s);
   return p.seq_rows || p.scorer != 0 ? launch_batch_modes(maps, p, st, fs, fp, num_sms, s)
                                      : launch_plain(maps, p, st, fs, fp, num_sms, s);
 }

@@ -102,7 +102,9 @@ enum {
   C_OFULL = C_MEMPTY + 2,
   C_OEMPTY = C_OFULL + kBatchWg,       // [2] per buffer
   C_CAND = C_OEMPTY + 2,               // [kBatchRows]
-  C_DRAIN = C_CAND + kBatchRows, C_DRAIN2 = C_DRAIN + 1, C_COUNT = C_DRAIN + 2
+  C_DRAIN = C_CAND + kBatchRows, C_DRAIN2 = C_DRAIN + 1,
+  C_XSTAT = C_DRAIN + 2, C_XO, C_XSEL,  // from the CTAs of a cluster: statistics, output, candidates
+  C_COUNT
 };
 
 // A batch: rows [row, row + nr). The CTA's first one is its own block index
@@ -121,7 +123,17 @@ __device__ __forceinline__ Item take_batch(const FusedStep& fs, const Dev& p, bo
 
 // HEUR, GLOB, GRAPH as in fused_kernel: a heuristic scorer instead of the
 // policy; the global token mode's per-row partial sums; device-counted steps.
-template <int D, int G, bool HEUR, bool GLOB, bool GRAPH>
+// CLUSTER: a row's tiles over the FusedStep::batch_cluster CTAs of a cluster,
+// one row per cluster. Rank k streams and scores tiles [k nT / C, (k + 1) nT / C);
+// through distributed shared memory the ranks exchange the row's softmax
+// statistics between the passes (each merges them in rank order), slices of
+// the output (rank k sums the k-th) and the lowest-ranked token (the last rank,
+// which holds slot n - 1, moves it). Rank 0 publishes the row's query and
+// statistics, once every rank has read the departing ones.
+// Bound by latency: 8 rows x 2049 tokens took 23.4 us a step on one CTA each (a
+// K and a V tile every 0.95 us, one after the other), 14.3 on clusters of 8: ~10
+// of launch, set-up and the row's serial parts, ~2 of exchanges, two tiles a rank.
+template <int D, int G, bool HEUR, bool GLOB, bool GRAPH, bool CLUSTER>
 __global__ void __launch_bounds__(kBatchThreads, 1)
     batch_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                  const __grid_constant__ CUtensorMap tmK16, const __grid_constant__ CUtensorMap tmV16, Dev p, Step st,
@@ -131,6 +143,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
   constexpr int kColO = 2 * NQ, kColStash = 2 * NQ + 64, kColZ = 256;
   static_assert(kColStash + GS * batch_tiles<G>() <= kColZ || GS == 0, "logits overlap the policy layer");
   static_assert(!GRAPH || (!HEUR && !GLOB), "device-counted steps: the plain step");
+  static_assert(!CLUSTER || !GLOB, "rows over clusters: per-row selection");
   if constexpr (GRAPH) {
     grid_dep_wait();  // the counter is the previous launch's
     const int t = *reinterpret_cast<volatile int*>(p.gcount);
@@ -154,7 +167,18 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
   float* red = reinterpret_cast<float*>(smem + L::RED);
 
   const int warp = threadIdx.x / kWarp, lane = threadIdx.x % kWarp;
-  const int n = st.n, nT = (n + kTok - 1) / kTok;
+  // this CTA's tokens of a row: n from the row's token toff on
+  const int csize = CLUSTER ? fs.batch_cluster : 1, crank = CLUSTER ? (int)(blockIdx.x % (unsigned)csize) : 0;
+  const int tiles = (st.n + kTok - 1) / kTok, tile0 = CLUSTER ? crank * tiles / csize : 0;
+  const int nT = CLUSTER ? (crank + 1) * tiles / csize - tile0 : tiles, toff = tile0 * kTok;
+  const int n = CLUSTER && crank < csize - 1 ? nT * kTok : st.n - toff;
+  // (rows on one CTA never use the second query slot's and the other rows'
+  // candidates' memory)
+  float* const xo = reinterpret_cast<float*>(smem + L::Q + L::QBYTES);                      // [csize][G D / csize]
+  float* const xst = reinterpret_cast<float*>(smem + L::CAND + 1024);                       // [csize][G][3]
+  unsigned* const xsel = reinterpret_cast<unsigned*>(smem + L::CAND + 2048);                // [csize][4]
+  static_assert(G * D * 4 <= L::QBYTES && 8 * G * 12 <= 1024 && 2048 + 8 * 16 <= kBatchRows * 4 * kBatchWg * 16,
+                "exchange areas");
   constexpr uint32_t kTileBytes = (uint32_t)D * kTok * 2;
 
   if (threadIdx.x == 0) {
@@ -187,6 +211,11 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     for (int s = 0; s < kBatchRows; ++s) mbar_init(&bar[C_CAND + s], 4 * (nT < kBatchWg ? nT : kBatchWg) + 1);
     mbar_init(&bar[C_DRAIN], 1);
     mbar_init(&bar[C_DRAIN2], 1);
+    if constexpr (CLUSTER) {
+      mbar_init(&bar[C_XSTAT], csize * G);
+      mbar_init(&bar[C_XO], csize * 4);
+      mbar_init(&bar[C_XSEL], csize);
+    }
     *abort = 0;
     for (int e = 0; e < kItemRing; ++e) items[4 * kItemRing + e] = 0;
     fence_mbar_init();
@@ -221,6 +250,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
   // the next launch's queue counter (this launch uses the other one)
   if (blockIdx.x == 0 && threadIdx.x == 0) fs.work[(fs.epoch + 1u) & 1u] = 0u;
   __syncthreads();
+  if constexpr (CLUSTER) cluster_sync();  // the ranks' barriers stand
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
@@ -241,6 +271,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
              DC_INB(p, ((long long)rq * p.w + st.slot) * G * D + G * D - 1, (long long)p.R * p.w * G * D, 102) &&
              DC_INB(p, ((long long)rq * p.w + st.slot_prev) * G * D, (long long)p.R * p.w * G * D, 103);
     };
+    const bool append = fs.k_new && crank == csize - 1;  // (the last rank holds slot st.n - 1)
     auto load_q = [&](int rq) {
       const uint4* cur = reinterpret_cast<const uint4*>(fs.q + ((rq / p.kvh) * p.qh + (rq % p.kvh) * G) * D);
       const uint4* prev = reinterpret_cast<const uint4*>(p.ring_q + ((size_t)rq * p.w + st.slot_prev) * G * D);
@@ -254,7 +285,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         qprev[u] = ld && st.has_prev ? prev[e] : make_uint4(0, 0, 0, 0);
         qdep[u] = ld && st.has_dep ? dep[e] : make_uint4(0, 0, 0, 0);
       }
-      if (fs.k_new && lane < 2 * VPR)
+      if (append && lane < 2 * VPR)
         kvn = (lane < VPR ? fs.k_new : fs.v_new)[(size_t)rq * VPR + lane % VPR];
       rstat = make_float4(0.f, 0.f, 0.f, 0.f);
       if (lane < 2 * G && ok)
@@ -275,7 +306,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         *reinterpret_cast<uint4*>(qk + sw128(h, kc & 7)) = qcur[u];
         *reinterpret_cast<uint4*>(qk + sw128(G + h, kc & 7)) = qprev[u];
         *reinterpret_cast<uint4*>(qk + sw128(2 * G + h, kc & 7)) = qdep[u];
-        ring_slot[e] = qcur[u];
+        if constexpr (!CLUSTER) ring_slot[e] = qcur[u];
       }
       if (lane < 2 * G) {
         float* w = qst + slot * 6 * G + 3 * G * sdep;
@@ -283,10 +314,10 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         w[G + sh] = rstat.w;
         w[2 * G + sh] = rstat.z;
       }
-      if (fs.k_new && DC_INB(p, n - 1, p.cap, 301) && DC_INB(p, rq, p.R, 301)) {
-        // the new pair into slot n - 1, with |v| and a clean state (as the append
+      if (append && DC_INB(p, st.n - 1, p.cap, 301) && DC_INB(p, rq, p.R, 301)) {
+        // the new pair into slot st.n - 1, with |v| and a clean state (as the append
         // kernel does it)
-        const size_t at = (size_t)rq * p.stride + (n - 1);
+        const size_t at = (size_t)rq * p.stride + (st.n - 1);
         if (lane < VPR) reinterpret_cast<uint4*>(p.K)[at * VPR + lane] = kvn;
         else if (lane < 2 * VPR) reinterpret_cast<uint4*>(p.V)[at * VPR + lane - VPR] = kvn;
         const uint32_t w4[4] = {kvn.x, kvn.y, kvn.z, kvn.w};
@@ -312,8 +343,12 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     auto take = [&](bool first) {
       int2 v = make_int2(-1, 0);
       if (lane == 0) {
-        const Item t = take_batch(fs, p, first);
-        v = make_int2(t.row, t.t0);
+        if constexpr (CLUSTER) {
+          if (first) v = make_int2((int)(blockIdx.x / (unsigned)csize), 1);
+        } else {
+          const Item t = take_batch(fs, p, first);
+          v = make_int2(t.row, t.t0);
+        }
       }
       v.x = __shfl_sync(0xffffffffu, v.x, 0);
       v.y = __shfl_sync(0xffffffffu, v.y, 0);
@@ -334,7 +369,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         const uint32_t aux_bytes = (vpass || GLOB) ? 0u : pos_bytes + sz_bytes;
         uint8_t* dst = smem + L::STAGE + s * kStageBytes;
         uint8_t* aux = smem + L::AUX + s * kAuxBytes;
-        const int y = rt * p.stride + j * kTok;
+        const int y = rt * p.stride + toff + j * kTok;
         issued = g + 1;
         if (!DC_INB(p, (long long)y + kTok - 1, (long long)p.R * p.stride, 104)) {
           mbar_arrive(&bar[C_FULL + s]);
@@ -374,7 +409,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         if (i + 1 < it.y) load_q(it.x + i + 1);
         // the last tile holds the new pair: its copies come after the writes of
         // it, whose latency the tiles before cover
-        if (fs.k_new) {
+        if (append) {
           if (elect_one()) ok = issue(it.x + i, false, 0, nT - 1);
           fence_proxy_async_global();
           __syncwarp();
@@ -391,6 +426,17 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         for (int i = 0; i < it.y && ok; ++i) ok = issue(it.x + i, true, 0, nT);
       ok = __all_sync(0xffffffffu, ok);
       it = nx;
+    }
+    if constexpr (CLUSTER) {
+      // every rank has read the departing query: the current one takes its slot
+      const int rq = (int)(blockIdx.x / (unsigned)csize);
+      if (crank == 0 && mbar_wait_cluster(&bar[C_XSTAT], 0, abort, p.dbg, 31u, (unsigned)rq) && q_ok(rq)) {
+        uint4* ring_slot = reinterpret_cast<uint4*>(p.ring_q + ((size_t)rq * p.w + st.slot) * G * D);
+#pragma unroll
+        for (int u = 0; u < QIT; ++u)
+          if (lane + u * kWarp < QCH) ring_slot[lane + u * kWarp] = qcur[u];
+      }
+      __syncwarp();
     }
     // every issued load must land before the CTA may exit
     if (elect_one())
@@ -518,10 +564,10 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
       nr = __shfl_sync(0xffffffffu, nr, 0);
       if (named_bar_or(1, kBatchEpi + kWarp, *abort != 0 || row0 < 0)) break;
       named_bar(1, kBatchEpi + kWarp);
-      for (int i = 0; !GLOB && fs.do_evict && n == Bsel + 1 && i < nr; ++i) {
+      for (int i = 0; !GLOB && fs.do_evict && st.n == Bsel + 1 && i < nr; ++i) {
         const int r = row0 + i;
         const size_t rbase = (size_t)r * (size_t)p.stride;
-        const bool ok = DC_INB(p, Bsel, p.stride, 116) && DC_INB(p, (long long)rbase + Bsel, (long long)p.R * p.stride, 116);
+        const bool ok = crank == csize - 1 && DC_INB(p, Bsel, p.stride, 116) && DC_INB(p, (long long)rbase + Bsel, (long long)p.R * p.stride, 116);
         SlotCopy mv{};
         if (ok) slot_load_settled(p, rbase + Bsel, lane, fs.write_scores, mv);
         mbar_wait(&bar[C_CAND + i], gr & 1, abort, p.dbg, 28u, (unsigned)r);
@@ -532,13 +578,37 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         // candidates (lowest key, then the latest position) is total
         const unsigned* cd = cand + i * 4 * kBatchWg * 4;
         const bool in = lane < 4 * kBatchWg && ((lane >> 2) + kBatchRows * kBatchWg - i) % kBatchWg < nT;
-        const int cs = in ? (int)cd[lane * 4 + 1] : -1;
-        const uint32_t ck = cs >= 0 ? cd[lane * 4] : 0xFFFFFFFFu;
-        const int cp = cs >= 0 ? (int)cd[lane * 4 + 2] : -1;
-        const uint32_t kmin = __reduce_min_sync(0xffffffffu, ck);
-        const int pmax = __reduce_max_sync(0xffffffffu, ck == kmin ? cp : -1);
-        const unsigned who = __ballot_sync(0xffffffffu, cs >= 0 && ck == kmin && cp == pmax);
-        const int fe = who ? __shfl_sync(0xffffffffu, cs, __ffs(who) - 1) : -1;
+        int cs = in ? (int)cd[lane * 4 + 1] : -1, cp = -1, fe = -1, pmax = -1;
+        uint32_t ck = 0xFFFFFFFFu, kmin = 0xFFFFFFFFu;
+        if (cs >= 0) {
+          ck = cd[lane * 4];
+          cp = (int)cd[lane * 4 + 2];
+        }
+        auto lowest = [&] {
+          kmin = __reduce_min_sync(0xffffffffu, ck);
+          pmax = __reduce_max_sync(0xffffffffu, ck == kmin ? cp : -1);
+          const unsigned who = __ballot_sync(0xffffffffu, cs >= 0 && ck == kmin && cp == pmax);
+          fe = who ? __shfl_sync(0xffffffffu, cs, __ffs(who) - 1) : -1;
+        };
+        lowest();
+        if constexpr (CLUSTER) {
+          // the ranks' candidates meet at the last rank, which moves; each rank
+          // sends its own once its tiles have been read (C_CAND)
+          if (lane == 0) {
+            const uint32_t at = cluster_addr(xsel + crank * 4, (uint32_t)csize - 1);
+            st_cluster(at, kmin);
+            st_cluster(at + 4, (unsigned)fe);
+            st_cluster(at + 8, (unsigned)pmax);
+            mbar_arrive_cluster(cluster_addr(&bar[C_XSEL], (uint32_t)csize - 1));
+          }
+          if (!ok) continue;
+          const bool all = mbar_wait_cluster(&bar[C_XSEL], 0, abort, p.dbg, 32u, (unsigned)r);
+          __syncwarp();
+          cs = all && lane < csize ? (int)xsel[lane * 4 + 1] : -1;
+          ck = cs >= 0 ? xsel[lane * 4] : 0xFFFFFFFFu;
+          cp = cs >= 0 ? (int)xsel[lane * 4 + 2] : -1;
+          lowest();
+        }
         if (ok && fe >= 0 && fe < Bsel && DC_INB(p, (long long)rbase + fe, (long long)p.R * p.stride, 117))
           slot_store(p, rbase + fe, lane, mv);
       }
@@ -586,7 +656,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         const int r = row0 + i;
         const int rs = rs0 + i, slot = rs % kQSlots;
         const float* wq = qst + slot * 6 * G;
-        const size_t rbase = (size_t)r * stride;
+        const size_t rbase = (size_t)r * stride + toff;
         // online softmax state; with batch_dual, even and odd tiles apart, as on
         // whole rows, where each of two warpgroups takes every other tile
         float m[G], l[G], u[G], m2[G], l2[G], u2[G];
@@ -633,7 +703,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
               const float mp = (st.has_prev && pos <= st.p_prev) ? 1.f : 0.f;
               const float md = (st.has_dep && pos <= st.p_dep) ? 1.f : 0.f;
               sz = window_update(sz, sp * mp, sd * md, zp * mp, zd * md);
-              if (slot_ok(r, ti, 105)) p.SZ[rbase + ti] = sz;
+              if (slot_ok(r, toff + ti, 105)) p.SZ[rbase + ti] = sz;
             }
           }
           scw[lt * kTok + tok] = S16[G - 1];
@@ -693,6 +763,26 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
             ll = __fmaf_rn(lw, f, ll);
             uu = __fmaf_rn(__fmaf_rn(lw, dm, redp[(w * G + h) * 3 + 2]), f, uu);
           }
+          if constexpr (CLUSTER) {
+            // to every rank, and the row's from all of them, in rank order
+            for (int k = 0; k < csize; ++k) {
+              const uint32_t at = cluster_addr(xst + (crank * G + h) * 3, (uint32_t)k);
+              st_cluster(at, __float_as_uint(mm));
+              st_cluster(at + 4, __float_as_uint(ll));
+              st_cluster(at + 8, __float_as_uint(uu));
+              mbar_arrive_cluster(cluster_addr(&bar[C_XSTAT], (uint32_t)k));
+            }
+            mbar_wait_cluster(&bar[C_XSTAT], 0, abort, p.dbg, 33u, (unsigned)r);
+            mm = kNoMax;
+            for (int k = 0; k < csize; ++k) mm = fmaxf(mm, xst[(k * G + h) * 3]);
+            ll = uu = 0.f;
+            for (int k = 0; k < csize; ++k) {
+              const float lk = xst[(k * G + h) * 3 + 1];
+              const float dm = __fmul_rn(__fsub_rn(xst[(k * G + h) * 3], mm), c), f = ex2(dm);
+              ll = __fmaf_rn(lk, f, ll);
+              uu = __fmaf_rn(__fmaf_rn(lk, dm, xst[(k * G + h) * 3 + 2]), f, uu);
+            }
+          }
           // H = ln l - ln 2 u / l
           float nl, hh;
           if (fs.batch_dual) {  // as whole rows do, from the hardware log2 and divide (l >= 1)
@@ -706,7 +796,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
           rst[(i * 3 + 0) * G + h] = mm;
           rst[(i * 3 + 1) * G + h] = nl;
           rst[(i * 3 + 2) * G + h] = hh;
-          if (DC_INB(p, (long long)r * p.w + st.slot, (long long)p.R * p.w, 109)) {
+          if (crank == 0 && DC_INB(p, (long long)r * p.w + st.slot, (long long)p.R * p.w, 109)) {
             reinterpret_cast<float4*>(p.ring_stats)[((size_t)r * p.w + st.slot) * G + h] = make_float4(mm, ll, hh, nl);
             p.hq[(size_t)r * G + h] = hh;
           }
@@ -737,7 +827,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
       int fi = 0, fj = wg - kBatchWg;  // before the warpgroup's first tile
       auto fetch = [&](float4& sz, int& pos, float& vn, float& ac) {
         advance(fi, fj);
-        const size_t at = (size_t)(row0 + fi) * stride + fj * kTok + tok;
+        const size_t at = (size_t)(row0 + fi) * stride + toff + fj * kTok + tok;
         if (fi < nr && DC_INB(p, (long long)at, (long long)p.R * p.stride, 107)) {
           if constexpr (!GLOB) {
             sz = p.SZ[at];
@@ -752,7 +842,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
       const float pos_den = (float)max(st.p_newest, 1);
       auto prep = [&](int pi, int j, unsigned tvj) {
         const int r = row0 + pi, lt = pi * nT + j;
-        const size_t rbase = (size_t)r * stride;
+        const size_t rbase = (size_t)r * stride + toff;
         const float4 sz = szA;
         const int pos = posA;
         const float vn = vnA, ac = acA;
@@ -802,7 +892,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         if constexpr (HEUR || GLOB) put_weights();
         if constexpr (GLOB) {
           // this row's share of the token's pooled sums
-          if (valid && slot_ok(r, i, 111)) {
+          if (valid && slot_ok(r, toff + i, 111)) {
             float a2 = 0.f;
 #pragma unroll
             for (int h = 0; h < G; ++h) a2 = fmaf(a[h], a[h], a2);
@@ -818,7 +908,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
         const float Zt = __fadd_rn(__fadd_rn(sz.z, zc), sz.w);
         const float St = __fadd_rn(__fadd_rn(sz.x, scur), sz.y);
         float x[5] = {mean, vn, var, Zt > 0.f ? St / Zt : 0.f, (float)pos / pos_den};
-        if (valid && slot_ok(r, i, 112)) {
+        if (valid && slot_ok(r, toff + i, 112)) {
           const size_t at = rbase + i;
           if (p.alpha_mode == 1) {
             x[0] = (ac_ahead ? ac : p.acc[at]) + mean;
@@ -884,13 +974,13 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
       // lowest-ranked token of the row so far (lower key, then later position)
       auto record = [&](int lt, int r, int j, float score, int pos) {
         const int i = j * kTok + tok;
-        if (i < n && slot_ok(r, i, 113)) {
+        if (i < n && slot_ok(r, toff + i, 113)) {
           scw[lt * kTok + tok] = score;
-          if (fs.write_scores) p.score[(size_t)r * stride + i] = score;
+          if (fs.write_scores) p.score[(size_t)r * stride + toff + i] = score;
           const uint32_t kk = score_key(score);
           if (ev_slot < 0 || kk < ev_key || (kk == ev_key && pos > ev_pos)) {
             ev_key = kk;
-            ev_slot = i;
+            ev_slot = toff + i;
             ev_pos = pos;
           }
         }
@@ -968,7 +1058,28 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bar[C_OEMPTY + ob]);
-            if (tok < D && DC_INB(p, (long long)((r / p.kvh) * p.qh + (r % p.kvh) * G) * D + (G - 1) * D + tok,
+            if constexpr (CLUSTER) {
+              // slice k of the row's outputs is rank k's to sum, in rank order
+              const int sl = G * D / csize;
+              if (tok < D)
+#pragma unroll
+                for (int h = 0; h < G; ++h) {
+                  const int e = h * D + tok;
+                  const float o = nT > 1 ? (o16[h] + odd[h]) + (o16[G + h] + odd[G + h]) : o16[h] + o16[G + h];
+                  st_cluster(cluster_addr(xo + crank * sl + e % sl, (uint32_t)(e / sl)), __float_as_uint(o));
+                }
+              __syncwarp();
+              if (lane < csize) mbar_arrive_cluster(cluster_addr(&bar[C_XO], (uint32_t)lane));
+              const bool all = mbar_wait_cluster(&bar[C_XO], 0, abort, p.dbg, 34u, (unsigned)rq);
+              __syncwarp();
+              const long long o0 = (long long)((r / p.kvh) * p.qh + (r % p.kvh) * G) * D + crank * sl;
+              if (all && DC_INB(p, o0 + sl - 1, (long long)(p.R / p.kvh) * p.qh * D, 115))
+                for (int e = tid; e < sl; e += kTeam) {
+                  float o = xo[e];
+                  for (int k = 1; k < csize; ++k) o += xo[k * sl + e];
+                  fs.out[o0 + e] = o;
+                }
+            } else if (tok < D && DC_INB(p, (long long)((r / p.kvh) * p.qh + (r % p.kvh) * G) * D + (G - 1) * D + tok,
                                   (long long)(p.R / p.kvh) * p.qh * D, 115)) {
               float* op = fs.out + ((r / p.kvh) * p.qh + (r % p.kvh) * G) * D;
 #pragma unroll
@@ -978,7 +1089,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
             // ---------------- argtop_B and prune of the row: several evictions
             // here (radix select over its scores: every warp's are in), one by
             // the mover
-            if (!GLOB && fs.do_evict && Bsel < n - 1) {
+            if (!GLOB && !CLUSTER && fs.do_evict && Bsel < n - 1) {
               mbar_wait(&bar[C_CAND + ci], gr & 1, abort, p.dbg, 30u, (unsigned)rq);
               __syncwarp();
               team_select_compact<kTeam>(p, r, n, Bsel, scw + ci * nT * kTok, tid, scr, sync);
@@ -993,6 +1104,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     }
   }
   __syncthreads();
+  if constexpr (CLUSTER) cluster_sync();  // no rank leaves while another may write to it
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
@@ -1009,26 +1121,35 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
   }
 }
 
-template <int D, int G, bool HEUR = false, bool GLOB = false, bool GRAPH = false>
+template <int D, int G, bool HEUR = false, bool GLOB = false, bool GRAPH = false, bool CLUSTER = false>
 static cudaError_t launch_batch_t(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                                   const FusedPolicy& fp, int num_sms, cudaStream_t s) {
   constexpr int kSmemBytes = BatchSmem<G>::BYTES;
+  const auto kernel = batch_kernel<D, G, HEUR, GLOB, GRAPH, CLUSTER>;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(batch_kernel<D, G, HEUR, GLOB, GRAPH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   const int rest = p.R - fs.batch_full * fs.batch_rows;
   const int items = fs.batch_full + (fs.batch_rest ? (rest + fs.batch_rest - 1) / fs.batch_rest : 0);
-  const int grid = items < num_sms ? items : num_sms;
-  if (!GRAPH)
-    return launch_pdl(batch_kernel<D, G, HEUR, GLOB, GRAPH>, dim3(grid), dim3(kBatchThreads), kSmemBytes, s, maps.k,
-                      maps.v, maps.k16, maps.v16, p, st, fs, fp);
-  batch_kernel<D, G, HEUR, GLOB, GRAPH><<<grid, kBatchThreads, kSmemBytes, s>>>(maps.k, maps.v, maps.k16, maps.v16, p,
-                                                                               st, fs, fp);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CLUSTER ? p.R * fs.batch_cluster : items < num_sms ? items : num_sms);
+  cfg.blockDim = dim3(kBatchThreads);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = s;
+  cudaLaunchAttribute la[2];
+  cfg.attrs = la;
+  if (!GRAPH) {
+    la[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    la[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (CLUSTER) {
+    la[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    la[cfg.numAttrs++].val.clusterDim = {(unsigned)fs.batch_cluster, 1, 1};
+  }
+  return cudaLaunchKernelEx(&cfg, kernel, maps.k, maps.v, maps.k16, maps.v16, p, st, fs, fp);
 }
 
 }  // namespace

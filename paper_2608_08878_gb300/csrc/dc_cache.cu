@@ -496,6 +496,7 @@ dc_status dc_cache_create(int layers, int kv_heads, int head_dim, int capacity, 
     }
     if (fe == cudaSuccess) {
       h->fused_ok = true;
+      if (h->xflag) dc::cluster_counts(p.clusters);
     } else {
       cudaGetLastError();
       h->fused_why = why;
@@ -669,9 +670,11 @@ dc_status graph_step(dc_cache* h, const void* q, const void* k_new, const void* 
   return DC_OK;
 }
 
-// Whether a decode step over n tokens would split the fused grid's last wave.
+// Whether a decode step over n tokens would split rows over CTAs (the fused
+// grid's last wave into halves, or every row over a cluster).
 bool tail_split_applies(dc_cache* h, int n, bool steady) {
   if (!h->xflag) return false;
+  if (steady && dc::fused_cluster(h->dev, n) > 1) return true;
   dc::FusedStep fs{};
   fs.xstats = h->xstats;
   fs.xo = h->xo;

@@ -69,6 +69,9 @@ struct Dev {
   // the departing query's exactly; and each sequence's move list
   // ([batch][1 + 2 stride]: count, then hole/mover pairs).
   int seq_rows, batch;
+  // few rows: clusters of 2, 4 and 8 CTAs of the fused step that the device holds
+  // at once (0: a row stays on one CTA)
+  int clusters[3];
   float4* gpart;
   float2* gring;
   int* gmoves;

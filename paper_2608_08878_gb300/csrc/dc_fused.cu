@@ -21,6 +21,14 @@ static int batch_tiles_of(int G) { return G == 8 ? batch_tiles<8>() : batch_tile
 
 void batch_items(const Dev& p, int n, int num_sms, FusedStep* fs) {
   const int nT = (n + kTok - 1) / kTok, fit = batch_tiles_of(p.G) / nT, cap = fit < kBatchRows ? fit : kBatchRows;
+  fs->batch_sms = num_sms;
+  fs->batch_cluster = fused_cluster(p, n);
+  if (fs->batch_cluster > 1) {
+    fs->batch_rows = 1;
+    fs->batch_full = p.R;
+    fs->batch_rest = fs->batch_dual = 0;
+    return;
+  }
   // as many rounds of full batches as all SMs can take, then one round of the
   // smallest batches that hold the rest: every SM gets the same number of rows,
   // to within one
@@ -30,7 +38,6 @@ void batch_items(const Dev& p, int n, int num_sms, FusedStep* fs) {
   fs->batch_rest = (rest + num_sms - 1) / num_sms;
   // (a few rows, or rows that ran in halves before: no whole-row order to keep)
   fs->batch_dual = p.R > 16 && !fused_pairs(p, n, num_sms) && !(2 * p.R <= num_sms && nT >= 12);
-  fs->batch_sms = num_sms;
 }
 
 bool batch_appends(const Dev& p, int num_sms) {
@@ -61,6 +68,26 @@ bool fused_pairs(const Dev& p, int n, int num_sms) {
   return waves2 * (2.0 * n + 410.0) < waves1 * (n + 350.0);
 }
 
+int fused_cluster(const Dev& p, int n) {
+  const int nT = (n + kTok - 1) / kTok;
+  if (p.seq_rows || p.rowlen) return 1;
+  // The largest cluster of which all rows' are resident at once (one wave more
+  // costs more than it gains: 16 rows x 2049 24.2 us a step on one CTA each, 27.8 in
+  // clusters of 8) and whose ranks get enough tiles to pay for ~3 us of
+  // exchanges and the cluster's launch. us a step, one CTA a row (two in
+  // halves from 30 tiles) -> clusters: of 8, 8 rows x 2049 23.4 -> 14.3, x 4097 31.9 ->
+  // 16.3, x 16385 83.5 -> 27.8, x 1025 15.7 -> 13.4; of 4, 24 x 1025 16.6 -> 14.5, 32 x 2049
+  // 24.3 -> 16.8, 32 x 8193 55.3 -> 29.4, but 8 x 601 11.9 -> 12.0, 24 x 601 12.6 -> 13.7; of
+  // 2, 64 x 2049 24.5 -> 20.6, 64 x 4097 40.7 -> 29.5, but 64 x 1025 16.9 -> 16.9, 64 x 601
+  // 13.0 -> 14.5.
+  const int least[3] = {10, 8, 16};
+  for (int i = 2; i >= 0; --i) {
+    const int c = 2 << i;
+    if (p.R <= p.clusters[i] && nT >= least[i] && (nT + c - 1) / c <= batch_tiles_of(p.G)) return c;
+  }
+  return 1;
+}
+
 bool fused_batches(const Dev& p, int n, int num_sms, bool steady) {
   // Rows of equal length whose logits fit on chip (6144 tokens, 2304 with eight
   // query heads). Batches measured faster than whole rows at every such size
@@ -76,6 +103,7 @@ bool fused_batches(const Dev& p, int n, int num_sms, bool steady) {
   // selection cuts through near-ties, keep the schedule that they had; steady
   // steps take the faster one.
   const int nT = (n + kTok - 1) / kTok;
+  if (steady && fused_cluster(p, n) > 1) return true;
   if (p.rowlen || nT > batch_tiles_of(p.G)) return false;
   if (fused_pairs(p, n, num_sms)) return true;
   return steady && !(4 * p.R <= num_sms && nT >= 30);

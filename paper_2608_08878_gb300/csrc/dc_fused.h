@@ -47,6 +47,7 @@ struct FusedStep {
   // batches of rows (batch_kernel): the first batch_full work items hold
   // batch_rows rows each, the others batch_rest; batch_rows 0: not on batches
   int batch_rows, batch_full, batch_rest;
+  int batch_cluster; // CTAs of a cluster that share a row (1: one CTA per row)
   int batch_sms;     // SMs (the whole-row schedule's CTAs)
   int batch_dual;    // 1: rows' statistics in the order of whole rows (see batch_kernel), 0: of row pairs
 };
@@ -93,6 +94,8 @@ void prepare_policy(const float* blob, int H, int layernorm, FusedPolicy* fp, st
 // part of the rule that dc_engine reports.
 bool fused_pairs(const Dev& p, int n, int num_sms);
 bool fused_batches(const Dev& p, int n, int num_sms, bool steady);
+// The CTAs a steady step there takes per row (1, or a cluster of 2, 4 or 8).
+int fused_cluster(const Dev& p, int n);
 // The division of the rows into work items there: see FusedStep.
 void batch_items(const Dev& p, int n, int num_sms, FusedStep* fs);
 // Whether such a step appends its new pairs in the kernel.
@@ -121,6 +124,12 @@ cudaError_t launch_batch_modes(const FusedMaps& maps, const Dev& p, const Step& 
 // Batches of rows (dc_batch.cu), FusedStep::batch_rows > 0.
 cudaError_t launch_fused_batch(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                               const FusedPolicy& fp, int num_sms, cudaStream_t s);
+// Clusters of 2, 4 and 8 CTAs of that kernel that the current device holds at once.
+void cluster_counts(int counts[3]);
+// Rows over clusters (dc_batch_cluster.cu), FusedStep::batch_cluster > 1, also
+// of device-counted steps.
+cudaError_t launch_batch_cluster(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
+                                 const FusedPolicy& fp, int num_sms, bool graph, cudaStream_t s);
 // Device-counted steps (dc_fused_graph.cu): st and fs.epoch are base values
 // that the kernel advances by Dev::gcount[0]; whole rows, halves or batches of
 // rows (as the plain step would take them), policy scorer, one eviction per step.

@@ -8,6 +8,7 @@ namespace dc {
 
 cudaError_t launch_fused_graph(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                                const FusedPolicy& fp, int num_sms, cudaStream_t s) {
+  if (fs.batch_rows && fs.batch_cluster > 1) return launch_batch_cluster(maps, p, st, fs, fp, num_sms, true, s);
   const int grid = fused_grid(p, fs, num_sms);
   const bool lg = st.n > fused_onchip_tokens(p.G);
 #define DC_FUSED_LAUNCH(D, G)                                                                                 \
