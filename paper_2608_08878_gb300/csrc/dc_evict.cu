@@ -222,50 +222,10 @@ __global__ void __launch_bounds__(kOneThreads) evict_one_kernel(Dev p, int n, in
   __shared__ int bslot[kOneThreads / kWarp];
   const int r = blockIdx.x, tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
   const size_t base = (size_t)r * p.stride;
-  const int* ps = p.pos + base;
   SlotCopy mv{};
   if (warp == 0 && DC_INB(p, B, p.stride, 206)) mv = slot_load(p, base + B, lane);
-  uint32_t key = 0xFFFFFFFFu;
-  int slot = -1;
-  // (k, i) ranks below the best so far? Positions are read only to break ties.
-  auto take = [&](uint32_t k, int i) {
-    if (slot < 0 || k < key || (k == key && ps[i] > ps[slot])) {
-      key = k;
-      slot = i;
-    }
-  };
-  const float4* s4 = reinterpret_cast<const float4*>(p.score + base);  // the stride is a multiple of 128 slots
-  for (int e = tid; e < (n >> 2); e += kOneThreads) {
-    const float4 v = s4[e];
-    take(score_key(v.x), 4 * e);
-    take(score_key(v.y), 4 * e + 1);
-    take(score_key(v.z), 4 * e + 2);
-    take(score_key(v.w), 4 * e + 3);
-  }
-  for (int i = (n & ~3) + tid; i < n; i += kOneThreads) take(score_key(p.score[base + i]), i);
-  // the warp's lowest-ranked candidate: the lowest key (no valid key is
-  // 0xFFFFFFFF), among equal keys the latest position
-  auto reduce = [&] {
-    const uint32_t kmin = __reduce_min_sync(0xffffffffu, slot >= 0 ? key : 0xFFFFFFFFu);
-    unsigned who = __ballot_sync(0xffffffffu, slot >= 0 && key == kmin);
-    if (__popc(who) > 1) {
-      const bool in = who >> lane & 1u;
-      const int at = in ? ps[slot] : -1, pmax = __reduce_max_sync(0xffffffffu, at);
-      who = __ballot_sync(0xffffffffu, in && at == pmax);
-    }
-    key = kmin;
-    slot = who ? __shfl_sync(0xffffffffu, slot, __ffs(who) - 1) : -1;
-  };
-  reduce();
-  if (lane == 0) {
-    bkey[warp] = key;
-    bslot[warp] = slot;
-  }
-  __syncthreads();
+  const int slot = lowest_ranked<kOneThreads>(p.score + base, p.pos + base, n, tid, bkey, bslot);
   if (warp > 0) return;
-  key = lane < kOneThreads / kWarp ? bkey[lane] : 0xFFFFFFFFu;
-  slot = lane < kOneThreads / kWarp ? bslot[lane] : -1;
-  reduce();
   // slot B fills the evicted slot
   if (slot >= 0 && slot < B) slot_store(p, base + slot, lane, mv);
 }

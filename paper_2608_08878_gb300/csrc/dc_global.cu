@@ -10,6 +10,12 @@
 // window sums, cumulative alpha, features and scores; beside it, the ring of
 // the last w queries' pooled terms per token (Dev::gring), which moves with
 // the tokens.
+//
+// After the rows' kernel the step is a chain of three short kernels (pooling,
+// selection, moves), bound by launch gaps and load latency: each is launched
+// while the one before runs and waits for it (programmatic dependent launch),
+// and the steady state's one eviction is an argmin. 256 rows x 411 tokens 35.5 ->
+// 27.8 us a step, 2 x 2049 37.7 -> 30.2, 64 x 16001 129.7 -> 121.2.
 #include "dc_common.cuh"
 #include "dc_kernels.h"
 #include "dc_select.cuh"
@@ -52,6 +58,8 @@ __global__ void __launch_bounds__(kFeatThreads) glob_feature_kernel(Dev p, Step 
   const int i = blockIdx.x * kFeatTok + t;
   for (int e = threadIdx.x; e < nblob; e += blockDim.x) wsm[e] = p.policy[e];
   float4 P = make_float4(0.f, 0.f, 0.f, 0.f);
+  grid_dep_wait();  // the rows' partial sums
+  grid_dep_launch();
   if (i < st.n) {
     const int S = p.seq_rows, r0 = grp * S / kFeatGroups, r1 = (grp + 1) * S / kFeatGroups;
     int l = r0 / p.kvh, g = r0 % p.kvh;
@@ -130,6 +138,8 @@ __global__ void __launch_bounds__(kSelThreads) glob_select_kernel(Dev p, int n, 
   const SelectScratch scr{hist, sh, wsum, best, best_slot};
   auto sync = [] { __syncthreads(); };
   const int b = blockIdx.x;
+  grid_dep_wait();
+  grid_dep_launch();
   const size_t base = (size_t)seq_row(p, b, 0, 0) * p.stride;
   int* moves = p.gmoves + (size_t)b * (1 + 2 * (size_t)p.stride);
   team_select_moves<kSelThreads>(p.score + base, p.pos + base, n, B, p.holes + base, moves, threadIdx.x, scr, sync);
@@ -139,6 +149,7 @@ __global__ void __launch_bounds__(kSelThreads) glob_select_kernel(Dev p, int n, 
 // move); the home row also moves the sequence's state.
 __global__ void __launch_bounds__(kMoveThreads) glob_compact_kernel(Dev p) {
   const int r = blockIdx.x;
+  grid_dep_wait();
   const int b = (r / p.kvh) % p.batch;
   const bool home = r == seq_row(p, b, 0, 0);
   const int* moves = p.gmoves + (size_t)b * (1 + 2 * (size_t)p.stride);
@@ -185,12 +196,12 @@ __global__ void __launch_bounds__(kMoveThreads) glob_compact_kernel(Dev p) {
 void launch_glob_features(const Dev& p, const Step& st, cudaStream_t s) {
   const dim3 grid((st.n + kFeatTok - 1) / kFeatTok, p.batch);
   const size_t smem = (size_t)((9 * p.hidden + 1 + 3) & ~3) * sizeof(float) + kFeatGroups * kFeatTok * sizeof(float4);
-  glob_feature_kernel<<<grid, kFeatThreads, smem, s>>>(p, st);
+  launch_pdl(glob_feature_kernel, grid, dim3(kFeatThreads), smem, s, p, st);
 }
 
 void launch_glob_evict(const Dev& p, int n, int B, cudaStream_t s) {
-  glob_select_kernel<<<p.batch, kSelThreads, 0, s>>>(p, n, B);
-  glob_compact_kernel<<<p.R, kMoveThreads, 0, s>>>(p);
+  launch_pdl(glob_select_kernel, dim3(p.batch), dim3(kSelThreads), 0, s, p, n, B);
+  launch_pdl(glob_compact_kernel, dim3(p.R), dim3(kMoveThreads), 0, s, p);
 }
 
 }  // namespace dc

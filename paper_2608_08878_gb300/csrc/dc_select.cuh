@@ -468,6 +468,57 @@ __device__ void team_select_compact(const Dev& p, int r, int n, int B, const flo
   team_select_compact_k<NT, false>(p, r, n, B, [&](int i) { return score_key(score[i]); }, tid, s, sync);
 }
 
+// The slot of a row's lowest-ranked token of n (lowest key, among equal keys the
+// latest position), found by the NT threads of a CTA; valid in its first warp, -1
+// without a valid key. `score` is 16-byte aligned; bkey and bslot: shared, one
+// entry per warp.
+template <int NT>
+__device__ int lowest_ranked(const float* score, const int* ps, int n, int tid, uint32_t* bkey, int* bslot) {
+  const int lane = tid % kWarp, warp = tid / kWarp;
+  uint32_t key = 0xFFFFFFFFu;
+  int slot = -1;
+  // (k, i) ranks below the best so far? Positions are read only to break ties.
+  auto take = [&](uint32_t k, int i) {
+    if (slot < 0 || k < key || (k == key && ps[i] > ps[slot])) {
+      key = k;
+      slot = i;
+    }
+  };
+  const float4* s4 = reinterpret_cast<const float4*>(score);
+  for (int e = tid; e < (n >> 2); e += NT) {
+    const float4 v = s4[e];
+    take(score_key(v.x), 4 * e);
+    take(score_key(v.y), 4 * e + 1);
+    take(score_key(v.z), 4 * e + 2);
+    take(score_key(v.w), 4 * e + 3);
+  }
+  for (int i = (n & ~3) + tid; i < n; i += NT) take(score_key(score[i]), i);
+  // the warp's lowest-ranked candidate: the lowest key (no valid key is
+  // 0xFFFFFFFF), among equal keys the latest position
+  auto reduce = [&] {
+    const uint32_t kmin = __reduce_min_sync(0xffffffffu, slot >= 0 ? key : 0xFFFFFFFFu);
+    unsigned who = __ballot_sync(0xffffffffu, slot >= 0 && key == kmin);
+    if (__popc(who) > 1) {
+      const bool in = who >> lane & 1u;
+      const int at = in ? ps[slot] : -1, pmax = __reduce_max_sync(0xffffffffu, at);
+      who = __ballot_sync(0xffffffffu, in && at == pmax);
+    }
+    key = kmin;
+    slot = who ? __shfl_sync(0xffffffffu, slot, __ffs(who) - 1) : -1;
+  };
+  reduce();
+  if (lane == 0) {
+    bkey[warp] = key;
+    bslot[warp] = slot;
+  }
+  __syncthreads();
+  if (warp > 0) return -1;
+  key = lane < NT / kWarp ? bkey[lane] : 0xFFFFFFFFu;
+  slot = lane < NT / kWarp ? bslot[lane] : -1;
+  reduce();
+  return slot;
+}
+
 // The same selection as team_select_compact without moving anything: writes
 // the compaction's (hole, mover) pairs to moves[1 + 2k], moves[2 + 2k] and
 // their count to moves[0] (for sequences whose rows all move alike). `holes`
@@ -482,40 +533,15 @@ __device__ void team_select_moves(const float* score, const int* ps, int n, int 
   }
   auto key = [&](int i) { return score_key(score[i]); };
   if (n == B + 1) {
-    uint32_t bk = 0xFFFFFFFFu;
-    int bs = -1;
-    for (int i = tid; i < n; i += NT) {
-      const uint32_t k = key(i);
-      if (bs < 0 || k < bk || (k == bk && ps[i] > ps[bs])) { bk = k; bs = i; }
-    }
-    auto better = [&](uint32_t ka, int sa, uint32_t kb, int sb) {
-      if (sb < 0) return false;
-      if (sa < 0) return true;
-      return kb < ka || (kb == ka && ps[sb] > ps[sa]);
-    };
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const uint32_t ok = __shfl_xor_sync(0xffffffffu, bk, off);
-      const int os = __shfl_xor_sync(0xffffffffu, bs, off);
-      if (better(bk, bs, ok, os)) { bk = ok; bs = os; }
-    }
-    const int lane = tid % kWarp, wid = tid / kWarp;
-    if (lane == 0) { s.best[wid] = bk; s.best_slot[wid] = bs; }
-    sync();
+    const int e = lowest_ranked<NT>(score, ps, n, tid, reinterpret_cast<uint32_t*>(s.best), s.best_slot);
     if (tid == 0) {
-      uint32_t fk = (uint32_t)s.best[0];
-      int e = s.best_slot[0];
-      for (int w = 1; w < NT / kWarp; ++w)
-        if (better(fk, e, (uint32_t)s.best[w], s.best_slot[w])) { fk = (uint32_t)s.best[w]; e = s.best_slot[w]; }
-      if (e >= 0 && e < B) {
-        moves[0] = 1;
+      const bool move = e >= 0 && e < B;
+      moves[0] = move;
+      if (move) {
         moves[1] = e;
         moves[2] = B;
-      } else {
-        moves[0] = 0;
       }
     }
-    sync();
     return;
   }
   int gt = 0;
