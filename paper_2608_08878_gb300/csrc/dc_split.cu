@@ -399,14 +399,17 @@ void launch_convert_sz(const Dev& p, int row0, int nrows, int which, double* dst
 // ---------------------------------------------------------------------------
 // Host launchers
 // ---------------------------------------------------------------------------
-// Per-row lengths: every row grew by T tokens.
+// Per-row lengths: every row grew by T tokens (after the append kernel, which
+// reads the lengths; the step kernel's set-up may run meanwhile).
 __global__ void rowlen_add_kernel(Dev p, int T) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r < p.R) p.rowlen[r] += T;
 }
 
 void launch_rowlen_add(const Dev& p, int T, cudaStream_t s) {
-  rowlen_add_kernel<<<(p.R + 255) / 256, 256, 0, s>>>(p, T);
+  launch_pdl(rowlen_add_kernel, dim3((p.R + 255) / 256), dim3(256), 0, s, p, T);
 }
 
 void launch_append(const Dev& p, const void* k, const void* v, int T, int n0, int seen0,
