@@ -13,10 +13,11 @@
 // each row on one warpgroup, then all V passes, so that one row's merge or
 // selection runs beside the tiles of the others; (2) three warpgroups take the
 // V tiles in turn, whatever row they belong to, and a warp of its own makes the
-// selections and moves. 623 us (89%; 256 rows: 19.7 -> 18.3). The V pass now takes
-// 1280 cycles a tile against 1200 of streaming; a fourth warpgroup would leave 96
-// registers a thread, and spills to an L1 that shared memory cut to 20 KB cost
-// more than it gave (1380 us).
+// selections and moves. 623 us (89%; 256 rows: 19.7 -> 18.3); 641 (86%) since rows'
+// sums keep whole rows' order (batch_dual). The V pass takes 1280 cycles a tile
+// against 1200 of streaming; a fourth warpgroup would leave 96 registers a thread,
+// and spills to an L1 that shared memory cut to 20 KB cost more than it gave (1380
+// us).
 //
 // A row's arithmetic and its order do not depend on the batch or on the tiles'
 // assignment: the statistics of a row come from one warpgroup in tile order
