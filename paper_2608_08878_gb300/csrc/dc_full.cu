@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(full_threads<G>(), full_ctas(G))
   uint4 kr[S::U];
   auto load = [&](const uint4* src, int t0, uint4 (&k)[S::U]) {
 #pragma unroll
-    for (int u = 0; u < S::U; ++u)  // past the end: the last token, weight 0
+    for (int u = 0; u < S::U; ++u)  // past the end: the last token again
       k[u] = ld_once(src + (size_t)min(t0 + u * S::TPW + grp, len - 1) * S::L);
   };
   constexpr int STEP = kFullWarps * S::TB;
@@ -218,11 +218,19 @@ __global__ void __launch_bounds__(full_threads<G>(), full_ctas(G))
     }
 #pragma unroll
     for (int i = 0; i < S::NV; ++i) {
-      const float w = valid && m[i] != -INFINITY ? ex2((x[i] - m[i]) * c) : 0.f;
+      // (a logit of -infinity has weight 0, also while the maximum is -infinity;
+      // a NaN, which the maximum passes over, is its weight's and the output's)
+      const float w = valid && x[i] != -INFINITY ? ex2((x[i] - m[i]) * c) : 0.f;
       l[i] += w;
       sp_[warp][grp * S::V + v0 + i] = w;
     }
     __syncwarp();
+    // past the end: zero values, as a weight of 0 makes NaN of an infinity
+    if (t0 + S::TB > len) {
+#pragma unroll
+      for (int u = 0; u < S::U; ++u)
+        if (t0 + u * S::TPW + grp >= len) vr[u] = make_uint4(0, 0, 0, 0);
+    }
 #pragma unroll
     for (int u = 0; u < S::U; ++u) {
       const float* pw = &sp_[warp][grp * S::V + u * G];
@@ -278,7 +286,8 @@ __global__ void __launch_bounds__(full_threads<G>(), full_ctas(G))
       if (grp == 0) *reinterpret_cast<float2*>(&so[warp][h * D + li * 8 + 2 * e]) = o;
     }
   __syncthreads();
-  // the split's result over its warps (a warp without tokens has m = -infinity)
+  // the split's result over its warps. A maximum of -infinity (no tokens, or no
+  // logit that is a number above it) counts 0 times: sums of 0 add nothing, NaN stays
   for (int e = tid; e < G * D; e += kFullThreads) {
     const int h = e / D;
     float M = -INFINITY;
@@ -287,8 +296,7 @@ __global__ void __launch_bounds__(full_threads<G>(), full_ctas(G))
     float num = 0.f, den = 0.f;
 #pragma unroll
     for (int w = 0; w < kFullWarps; ++w) {
-      if (sml[w][h][0] == -INFINITY) continue;
-      const float f = ex2((sml[w][h][0] - M) * c);
+      const float f = sml[w][h][0] == -INFINITY ? 0.f : ex2((sml[w][h][0] - M) * c);
       den += sml[w][h][1] * f;
       num += so[w][e] * f;
     }
@@ -311,8 +319,7 @@ __global__ void __launch_bounds__(full_threads<G>(), full_ctas(G))
     float num = 0.f, den = 0.f;
     for (int s = 0; s < nsplit; ++s) {
       const float ms = ld_peer(&cml[h][0], s);
-      if (ms == -INFINITY) continue;
-      const float f = ex2((ms - M) * c);
+      const float f = ms == -INFINITY ? 0.f : ex2((ms - M) * c);
       den += ld_peer(&cml[h][1], s) * f;
       num += ld_peer(&co[e], s) * f;
     }
