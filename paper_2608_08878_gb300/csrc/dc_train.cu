@@ -11,7 +11,7 @@
 //
 // (expand the product: the subset a has probability prod_{a} p_i prod_{not a}
 // (1 - p_i)). u is chosen so that E[S] is B to a tenth of a standard deviation
-// (safeguarded Newton steps on the monotone E[S]): P(S = B) is then of the order
+// (safeguarded Newton steps on the monotone E[S], see next_shift): P(S = B) is then of the order
 // of 1 / (1 + sd), and an inverse discrete Fourier transform of the
 // characteristic function phi(w) = prod_i (1 - p_i + p_i e^{iw}) gives it
 // (Fernandez and Williams 2010; Hong 2013):
@@ -82,6 +82,50 @@ __device__ __forceinline__ void logistic(float x, float& p, float& q, float& e) 
   q = x > 0.f ? small : inv;
 }
 
+// The search for the shift: E[S] < B at u = lo, > B at u = hi. Where equal values
+// of 1e10 and more straddle the cut (a row padded with a large negative number, B
+// beyond the items before the padding), no double near the root brings E[S] to B:
+// fp32 values around -u are so far apart there that E[S] varies with one of them
+// alone. Then that value is split off, u = tie + v with v in [lo, hi] instead.
+struct Search {
+  double u, lo, hi;
+  float tie;  // minus that value; 0 while u is a number of its own
+};
+
+constexpr int kNewtonSteps = 64;  // only halving after these
+constexpr int kMaxSteps = 200;    // (147 at most: 64, 32 halvings between fp32 numbers, 31 below 2^20, 20 of v)
+
+// A float's bits in the order of the numbers, as a signed integer, and back.
+__device__ __forceinline__ int ordered(int bits) { return bits ^ ((bits >> 31) & 0x7fffffff); }
+
+// The next shift, from d = B - E[S] and the variance at this one.
+__device__ __forceinline__ void next_shift(Search& s, int step, float d, float var) {
+  if (d > 0.f) s.lo = s.u;
+  else s.hi = s.u;
+  // From 2^33 on fp32 numbers are at least 2^-24 |u| >= 512 apart, and E[S] differs
+  // from whole numbers by 0.05 only within ln(25599 / 0.05) < 14 of one.
+  const double width = s.hi - s.lo, mag = fabs(s.u);
+  if (s.tie == 0.f && mag >= 8589934592.0 && width <= fmax(256.0, mag * 0x1p-32)) {
+    s.tie = (float)(0.5 * (s.lo + s.hi));
+    s.lo = -64.0;
+    s.hi = 64.0;
+    s.u = 0.0;
+    return;
+  }
+  // a Newton step where it stays inside the bracket, else its middle, counted in
+  // fp32 numbers while it is wide (the values may span many orders of magnitude)
+  double nu = s.u + (double)(d / var);
+  if (!(step < kNewtonSteps && nu > s.lo && nu < s.hi)) {
+    nu = 0.5 * (s.lo + s.hi);
+    if (width > 1048576.0) {
+      const long long a = ordered(__float_as_int((float)s.lo)), b = ordered(__float_as_int((float)s.hi));
+      const double m = (double)__int_as_float(ordered((int)((a + b) >> 1)));
+      if (m > s.lo && m < s.hi) nu = m;
+    }
+  }
+  s.u = nu;
+}
+
 // One CTA per row. Bound by latency: a handful of block-wide reductions over a
 // row held in shared memory, in short loops (unrolled over registers, the code
 // ran once per row out of a cold instruction cache: 44 us against 22, caches
@@ -126,8 +170,13 @@ __global__ void __launch_bounds__(kLzMaxWarps* kWarp) pl_logz_kernel(const float
     rs[warp][0] = mx; rs[warp][1] = mn; rs[warp][2] = sum; rs[warp][3] = cnt;
   }
   __syncthreads();
-  // thread 0's part of the search: u in [lo, hi], E[S] < B at lo and > B at hi
-  double u = 0.0, lo = 0.0, hi = 0.0;
+  Search srch = {0.0, 0.0, 0.0, 0.f};  // (thread 0's)
+  // u in three numbers for all threads: whole, and a float part with the rest
+  auto publish = [&] {
+    sh_uh = srch.tie != 0.f ? srch.tie : (float)srch.u;
+    sh_ul = (float)(srch.tie != 0.f ? srch.u : srch.u - (double)sh_uh);
+    sh_u = (double)srch.tie + srch.u;
+  };
   if (tid == 0) {
     for (int w = 1; w < nw; ++w) {
       mx = max_nan(mx, rs[w][0]);
@@ -139,15 +188,14 @@ __global__ void __launch_bounds__(kLzMaxWarps* kWarp) pl_logz_kernel(const float
     const int st = !(mx < INFINITY) ? 3 : cnt < (float)B ? 1 : cnt == (float)B ? 2 : 0;
     if (st == 0) {
       const float rest = cnt - (float)B;
-      lo = (double)(logf((float)B / cnt) - 1.f) - (double)mx;
-      hi = (double)(1.f - logf(rest / cnt)) - (double)mn;
-      u = (double)(logf((float)B / rest) - sum / cnt);
-      u = u < lo ? lo : u > hi ? hi : u;
+      srch.lo = (double)(logf((float)B / cnt) - 1.f) - (double)mx;
+      srch.hi = (double)(1.f - logf(rest / cnt)) - (double)mn;
+      const double u = (double)(logf((float)B / rest) - sum / cnt);
+      srch.u = u < srch.lo ? srch.lo : u > srch.hi ? srch.hi : u;
+      if (u != u) srch.u = 0.5 * (srch.lo + srch.hi);  // (partial sums of both infinities)
     }
     sh_state = st;
-    sh_u = u;
-    sh_uh = (float)u;
-    sh_ul = (float)(u - (double)sh_uh);
+    publish();
   }
   __syncthreads();
   const int state = sh_state;
@@ -156,7 +204,7 @@ __global__ void __launch_bounds__(kLzMaxWarps* kWarp) pl_logz_kernel(const float
     return;
   }
   // ---- the shift: |E[S] - B| <= sd / 10 (or 1 / 20)
-  for (int step = 0; state == 0 && step < 400; ++step) {
+  for (int step = 0; state == 0 && step < kMaxSteps; ++step) {
     const float uh = sh_uh, ul = sh_ul;
     float fp = 0.f, fv = 0.f;
 #pragma unroll 4
@@ -184,14 +232,8 @@ __global__ void __launch_bounds__(kLzMaxWarps* kWarp) pl_logz_kernel(const float
         if (fabsf(d) <= 0.1f * fmaxf(sqrtf(fv), 0.5f)) {
           sh_state = 4;
         } else {
-          if (d > 0.f) lo = u;
-          else hi = u;
-          // a Newton step where it stays inside the bracket, else its middle
-          const double nu = u + (double)(d / fv);
-          u = nu > lo && nu < hi ? nu : 0.5 * (lo + hi);
-          sh_u = u;
-          sh_uh = (float)u;
-          sh_ul = (float)(u - (double)sh_uh);
+          next_shift(srch, step, d, fv);
+          publish();
         }
       }
     }
@@ -231,6 +273,7 @@ __global__ void __launch_bounds__(kLzMaxWarps* kWarp) pl_logz_kernel(const float
     pl = lane < nw ? rs[lane][1] : 0.f;
     warp_add2(ph, pl);
     np = warp_sum(lane < nw ? rs[lane][2] : 0.f);
+    if (!(fabsf(ph) < INFINITY)) pl = 0.f;  // past the fp32 range: infinite, not NaN
     A = (double)ph + (double)pl + (double)(np - (float)B) * sh_u;
     if (state == 2 && lane == 0) out[row] = (float)A;  // (np = B: the shift takes no part)
   }
