@@ -1,8 +1,6 @@
 // dc_batch_cluster.cu -- instantiations of the fused step with few rows, each
 // over a thread-block cluster (dc_batch_kernel.cuh): the policy scorer, also on
 // device-counted steps, and the heuristic scorers.
-#include <mutex>
-
 #include "dc_batch_kernel.cuh"
 
 namespace dc {
@@ -10,12 +8,12 @@ namespace dc {
 void cluster_counts(int counts[3]) {
   // asked once per device (how many clusters fit depends on how its SMs are
   // grouped); every instantiation takes a whole SM per CTA, so one stands for all
-  constexpr int kDevices = 64;
-  static std::once_flag once[kDevices];
-  static int resident[kDevices][3];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) dev = 0;
-  std::call_once(once[dev], [&] {
+  struct Counts {
+    int of[3];
+  };
+  static PerDevice<Counts> resident;
+  const Counts c = resident.get([] {
+    Counts r = {};
     const auto kernel = batch_kernel<128, 4, false, false, false, true>;
     constexpr int kSmemBytes = BatchSmem<4>::BYTES;
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
@@ -29,11 +27,12 @@ void cluster_counts(int counts[3]) {
     for (int i = 0; i < 3; ++i) {
       cfg.gridDim = dim3(2u << i);
       la[0].val.clusterDim = {2u << i, 1, 1};
-      if (cudaOccupancyMaxActiveClusters(&resident[dev][i], kernel, &cfg) != cudaSuccess) resident[dev][i] = 0;
+      if (cudaOccupancyMaxActiveClusters(&r.of[i], kernel, &cfg) != cudaSuccess) r.of[i] = 0;
     }
     cudaGetLastError();  // a size that the device refuses is not used
+    return r;
   });
-  for (int i = 0; i < 3; ++i) counts[i] = resident[dev][i];
+  for (int i = 0; i < 3; ++i) counts[i] = c.of[i];
 }
 
 cudaError_t launch_batch_cluster(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,

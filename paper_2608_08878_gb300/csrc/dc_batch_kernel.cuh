@@ -1127,12 +1127,8 @@ static cudaError_t launch_batch_t(const FusedMaps& maps, const Dev& p, const Ste
                                   const FusedPolicy& fp, int num_sms, cudaStream_t s) {
   constexpr int kSmemBytes = BatchSmem<G>::BYTES;
   const auto kernel = batch_kernel<D, G, HEUR, GLOB, GRAPH, CLUSTER>;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(kernel, kSmemBytes); e != cudaSuccess) return e;
   const int rest = p.R - fs.batch_full * fs.batch_rows;
   const int items = fs.batch_full + (fs.batch_rest ? (rest + fs.batch_rest - 1) / fs.batch_rest : 0);
   cudaLaunchConfig_t cfg = {};

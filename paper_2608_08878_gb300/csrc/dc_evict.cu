@@ -3,6 +3,7 @@
 // one CTA per row, ranks the row and lists its holes and movers; a move
 // kernel, spread over the whole GPU, copies the movers into the holes.
 #include "dc_common.cuh"
+#include "dc_device.h"
 #include "dc_kernels.h"
 #include "dc_select.cuh"
 
@@ -243,13 +244,9 @@ void launch_evict(const Dev& p, int n, int B, cudaStream_t s) {
     evict_one_kernel<<<p.R, kOneThreads, 0, s>>>(p, n, B);
     return;
   }
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(evict_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kSmemKeys * (int)sizeof(uint32_t)) != cudaSuccess)
-      return;  // the launch below then fails and the caller reports the error
-    attr = true;
-  }
+  static SmemLimit limit;
+  if (limit.raise(evict_select_kernel, kSmemKeys * (int)sizeof(uint32_t)) != cudaSuccess)
+    return;  // (the caller reports the error)
   const int smem_keys = n <= kSmemKeys ? n : 0;
   evict_select_kernel<<<p.R, kEvictThreads, (size_t)smem_keys * sizeof(uint32_t), s>>>(p, n, B, smem_keys);
   const int mm = max_moves(n, B);

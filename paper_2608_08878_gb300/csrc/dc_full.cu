@@ -18,9 +18,8 @@
 // in global memory, no second kernel.
 // 64 rows x 8192 tokens, D 128, G 4: 182 -> 56 us (40 us at the copy
 // bandwidth), and a smaller error against 64 bits (4.5e-7 -> 2.8e-7).
-#include <mutex>
-
 #include "dc_common.cuh"
+#include "dc_device.h"
 #include "dc_kernels.h"
 
 namespace dc {
@@ -348,23 +347,23 @@ void full_t(const Dev& p, int n, int num_sms, const void* q, float* out, cudaStr
   cfg.attrs = la;
   cfg.numAttrs = 1;
   // resident clusters of each size, asked once per device
-  constexpr int kDevices = 64;
-  static std::once_flag once[kDevices];
-  static int active_on[kDevices][kMaxSplits + 1];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) dev = 0;
-  int* const active = active_on[dev];
-  std::call_once(once[dev], [&] {
+  struct Counts {
+    int of[kMaxSplits + 1];
+  };
+  static PerDevice<Counts> resident;
+  const Counts active = resident.get([&] {
+    Counts r = {};
     const bool large = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     for (int k = 1; k <= kMaxSplits; ++k) {
       int m = 0;
       cfg.gridDim = dim3(k);
       la[0].val.clusterDim = {(unsigned)k, 1, 1};
       if ((k > 8 && !large) || cudaOccupancyMaxActiveClusters(&m, kernel, &cfg) != cudaSuccess) m = 0;
-      active[k] = m;
+      r.of[k] = m;
     }
     cudaGetLastError();  // a size that the device refuses is not used
-    if (active[1] == 0) active[1] = full_ctas(G) * num_sms;
+    if (r.of[1] == 0) r.of[1] = full_ctas(G) * num_sms;
+    return r;
   });
   const int tiles = (n + 127) / 128;
   // ns per token of a CTA at its share of the bandwidth
@@ -372,8 +371,8 @@ void full_t(const Dev& p, int n, int num_sms, const void* q, float* out, cudaStr
   int nsplit = 1, chunk = tiles * 128;
   double best = 0.0;
   for (int k = 1; k <= kMaxSplits && k <= tiles; ++k) {
-    if (active[k] == 0) continue;
-    const int c = (tiles + k - 1) / k * 128, waves = (p.R + active[k] - 1) / active[k];
+    if (active.of[k] == 0) continue;
+    const int c = (tiles + k - 1) / k * 128, waves = (p.R + active.of[k] - 1) / active.of[k];
     const double t = waves * (token_ns * c + 3000.0);
     if (best == 0.0 || t < best) {
       best = t;

@@ -62,6 +62,7 @@
 #include <cuda.h>
 
 #include "dc_common.cuh"
+#include "dc_device.h"
 #include "dc_fused.h"
 #include "dc_kernels.h"
 #include "dc_select.cuh"
@@ -1300,13 +1301,10 @@ template <int D, int G, bool LONG, bool FULL = false, bool HEUR = false, bool GL
 static cudaError_t launch_t(const FusedMaps& maps, const Dev& p, const Step& st, const FusedStep& fs,
                             const FusedPolicy& fp, int grid, cudaStream_t s) {
   constexpr int kSmemBytes = Smem<G>::BYTES;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, GRAPH>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemLimit limit;
+  if (cudaError_t e = limit.raise(fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, GRAPH>, kSmemBytes);
+      e != cudaSuccess)
+    return e;
   if (fs.half_rows == 0 && !GRAPH)
     return launch_pdl(fused_kernel<D, G, LONG, FULL, HEUR, GLOB, PERROW, GRAPH>, dim3(grid), dim3(kThreads),
                       kSmemBytes, s, maps.k, maps.v, maps.k16, maps.v16, p, st, fs, fp);
