@@ -381,6 +381,12 @@ dc_status dc_debug_bounds_selftest(unsigned* result, void* stream);
  * DC_ERR_STATE. */
 dc_status dc_debug_corrupt_guard(dc_cache* h);
 
+/* How the fused engine would divide the rows of a decode step over n tokens per
+ * row (n <= 0: the next one): rows of a batch and CTAs of a cluster that shares
+ * one (0, 0: whole rows), and how many whole rows are split in halves. All 0 on
+ * the split engine. Host-only. */
+dc_status dc_debug_schedule(dc_cache* h, int n, int* batch_rows, int* cluster, int* half_rows);
+
 /* Message of the last error on the handle (or of the last failed create when
  * h is NULL). Valid until the next call on the handle. */
 const char* dc_last_error(const dc_cache* h);

@@ -600,8 +600,20 @@ int effective_budget(const dc_cache* h, int budget, int n_cached, long long seen
 // for dc_step and dc_decode_step.
 bool steady_step(const dc_cache* h, int n, long long seen) { return n - 1 <= effective_budget(h, 0, n, seen); }
 
-// Arguments of one fused launch; enables the half-row tail split when the
-// handle has exchange buffers and the step qualifies.
+// How a fused launch over n tokens divides the rows among the CTAs: batches or
+// clusters, or whole rows with some of them (or all) in halves, where the handle
+// has exchange buffers and the step qualifies. `full`: attention alone.
+void plan_rows(const dc_cache* h, int n, bool steady, bool full, dc::FusedStep* fs) {
+  fs->xstats = h->xstats;
+  fs->xo = h->xo;
+  fs->xsel = h->xsel;
+  fs->xflag = h->xflag;
+  fs->xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
+  fs->half_rows = (h->xflag && !h->per_row) ? dc::fused_half_rows(h->dev, n, *fs, h->num_sms, steady) : 0;
+  if (!full && dc::fused_batches(h->dev, n, h->num_sms, steady)) dc::batch_items(h->dev, n, h->num_sms, fs);
+}
+
+// Arguments of one fused launch.
 dc::FusedStep fused_args(dc_cache* h, const dc::Step& st, const void* q, float* out, int do_evict, int B,
                          int write_scores, bool full = false) {
   dc::FusedStep fs{};
@@ -610,15 +622,8 @@ dc::FusedStep fused_args(dc_cache* h, const dc::Step& st, const void* q, float* 
   fs.do_evict = do_evict;
   fs.B = B;
   fs.write_scores = write_scores;
-  fs.xstats = h->xstats;
-  fs.xo = h->xo;
-  fs.xsel = h->xsel;
-  fs.xflag = h->xflag;
-  fs.xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
   fs.work = h->work;
-  const bool steady = !full && steady_step(h, st.n, h->seen + 1);
-  fs.half_rows = (h->xflag && !h->per_row) ? dc::fused_half_rows(h->dev, st.n, fs, h->num_sms, steady) : 0;
-  if (!full && dc::fused_batches(h->dev, st.n, h->num_sms, steady)) dc::batch_items(h->dev, st.n, h->num_sms, &fs);
+  plan_rows(h, st.n, !full && steady_step(h, st.n, h->seen + 1), full, &fs);
   // launch epoch: the queue counter is work[epoch & 1]; exchange flags hold
   // epoch * 4 + phase (1..3), so a flag left by an earlier launch never matches
   fs.epoch = ++h->epoch;
@@ -637,28 +642,19 @@ bool kernel_appends(const dc_cache* h, int n) {
 // host's mirror of the step state stays at the base until the mode ends.
 dc_status graph_step(dc_cache* h, const void* q, const void* k_new, const void* v_new, float* out, int budget) {
   if (budget > 0 && budget != h->budget) return fail(h, DC_ERR_INVALID_ARG, "graph mode keeps the configured budget");
-  const bool batches = dc::fused_batches(h->dev, h->gstep.n, h->num_sms, true);
-  const bool appends = batches && dc::batch_appends(h->dev, h->num_sms);
-  if (!appends) {
-    Phase ph(h, DC_PHASE_APPEND, 1);
-    dc::launch_append(h->dev, k_new, v_new, 1, h->n, h->gstep.p_newest, h->stream);
-  }
   dc::FusedStep fs{};
   fs.q = (const __nv_bfloat16*)q;
   fs.out = out;
   fs.do_evict = 1;
   fs.B = h->budget;
-  fs.xstats = h->xstats;
-  fs.xo = h->xo;
-  fs.xsel = h->xsel;
-  fs.xflag = h->xflag;
-  fs.xslots = h->xflag ? (int)std::min<long long>(h->dev.R, h->num_sms) + 1 : 0;
   fs.work = h->work;
-  fs.half_rows = h->xflag ? dc::fused_half_rows(h->dev, h->gstep.n, fs, h->num_sms, true) : 0;
-  if (batches) dc::batch_items(h->dev, h->gstep.n, h->num_sms, &fs);
-  if (appends) {
+  plan_rows(h, h->gstep.n, true, false, &fs);
+  if (fs.batch_rows && dc::batch_appends(h->dev, h->num_sms)) {
     fs.k_new = (const uint4*)k_new;
     fs.v_new = (const uint4*)v_new;
+  } else {
+    Phase ph(h, DC_PHASE_APPEND, 1);
+    dc::launch_append(h->dev, k_new, v_new, 1, h->n, h->gstep.p_newest, h->stream);
   }
   fs.epoch = h->gepoch;
   cudaError_t e;
@@ -1232,6 +1228,18 @@ dc_status dc_debug_corrupt_guard(dc_cache* h) {
   // handle owns, outside every buffer
   char* at = (char*)h->allocs[0].base + kGuardBytes + h->allocs[0].bytes;
   DC_CUDA(h, cudaMemsetAsync(at, (unsigned char)~kGuardByte, 1, h->stream));
+  return DC_OK;
+}
+
+dc_status dc_debug_schedule(dc_cache* h, int n, int* batch_rows, int* cluster, int* half_rows) {
+  DC_CHECK_HANDLE(h);
+  if (!batch_rows || !cluster || !half_rows) return fail(h, DC_ERR_INVALID_ARG, "NULL pointer");
+  const int nn = n > 0 ? n : h->n + 1;
+  dc::FusedStep fs{};
+  if (use_fused(h, nn)) plan_rows(h, nn, steady_step(h, nn, h->seen + 1), false, &fs);
+  *batch_rows = fs.batch_rows;
+  *cluster = fs.batch_rows ? fs.batch_cluster : 0;
+  *half_rows = fs.half_rows;
   return DC_OK;
 }
 

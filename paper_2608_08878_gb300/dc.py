@@ -35,7 +35,7 @@ EXPORTS = ["dc_config_default", "dc_cache_create", "dc_cache_destroy", "dc_polic
            "dc_noalloc_last_error", "dc_pl_log_partition", "dc_gumbel_top_b", "dc_train_last_error",
            "dc_set_row_budgets", "dc_get_row_lengths", "dc_wait_selftest", "dc_selftest_last_error",
            "dc_set_graph_mode", "dc_debug_fail_alloc", "dc_debug_checks", "dc_debug_bounds_selftest",
-           "dc_debug_corrupt_guard"]
+           "dc_debug_corrupt_guard", "dc_debug_schedule"]
 PHASES = ["append", "attend", "stats", "score", "combine", "evict", "full"]
 
 
@@ -100,6 +100,7 @@ def lib():
             L.dc_debug_checks.argtypes = []
             L.dc_debug_bounds_selftest.argtypes = [P, P]
             L.dc_debug_corrupt_guard.argtypes = [P]
+            L.dc_debug_schedule.argtypes = [P, I, C.POINTER(I), C.POINTER(I), C.POINTER(I)]
             L.dc_selftest_last_error.argtypes = []
             L.dc_selftest_last_error.restype = C.c_char_p
             L.dc_get_length.argtypes = [P, C.POINTER(I), C.POINTER(C.c_longlong)]
@@ -407,6 +408,12 @@ class DistillCache:
     def debug_corrupt_guard(self) -> None:
         """Debug builds: damages a guard region so the next sync() must fail."""
         self._check(lib().dc_debug_corrupt_guard(self._h))
+
+    def debug_schedule(self, n: int = 0) -> dict:
+        """How the fused engine would divide the rows of a step over n tokens (see dc_debug_schedule)."""
+        x = [C.c_int() for _ in range(3)]
+        self._check(lib().dc_debug_schedule(self._h, n, *(C.byref(v) for v in x)))
+        return dict(zip(("batch_rows", "cluster", "half_rows"), (v.value for v in x)))
 
     def set_graph_mode(self, enable: bool = True) -> None:
         """Device-counted steps: a CUDA graph captured from one step() replays
