@@ -323,8 +323,9 @@ dc_status dc_sync(dc_cache* h);
  * while loading the module).
  * DC_ERR_CAPACITY if rows * group * (head_dim + 4) * 4 > 16 MiB;
  * DC_ERR_INVALID_ARG for bad shapes (head_dim 64 or 128, group 1, 2, 4 or 8,
- * 1 <= rows <= 65535, n >= 1). Make the first call on a device before any
- * stream capture. Calls may overlap on the GPU. Asynchronous on `stream`;
+ * 1 <= rows <= 65535, n >= 1). As softmax has it, a NaN key makes its row's
+ * output NaN and a logit of -infinity has no weight. Make the first call on a
+ * device before any stream capture. Calls may overlap on the GPU. Asynchronous on `stream`;
  * dc_noalloc_last_error() describes a failure. */
 dc_status dc_attend_noalloc(const void* q, const void* k, const void* v, int rows, int n,
                             int head_dim, int group, float* out, void* stream);
@@ -403,7 +404,8 @@ const char* dc_last_error(const dc_cache* h);
  * that a sum of independent Bernoulli variables is B (their characteristic
  * function, inverted at a few points), after a shift that centres the sum on B;
  * |error| <= 2 L 2^-24 (|log Z| + max |s| / tau) + L 2^-21. A score of
- * -infinity takes no part; NaN and +infinity give NaN. Needs
+ * -infinity takes no part; NaN and +infinity give NaN; sums past the fp32 range
+ * are infinite. Needs
  * 1 <= B <= L, rows <= 65535, B <= 25599, tau > 0;
  * else DC_ERR_INVALID_ARG (message in dc_train_last_error()). */
 dc_status dc_pl_log_partition(const float* scores, int rows, int L, int B, float tau, float* out,

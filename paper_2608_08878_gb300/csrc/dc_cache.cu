@@ -267,8 +267,11 @@ bool use_fused(const dc_cache* h, int n) {
   // two CTAs (rows of 12 tiles or more, at most half as many rows as SMs: ~16
   // us with the exchange, 0.75 us per 128 tokens); the split engine spreads
   // the rows over the GPU but costs ~57 us of launches plus ~0.55 ns per
-  // token-row (all measured on Mistral-7B head shapes). The split engine wins
-  // only for a few very long rows.
+  // token-row (all measured on Mistral-7B head shapes). By these estimates the
+  // split engine wins for a few very long rows only. They are those of whole rows
+  // and halves: a steady step of few rows runs on clusters, which beat both (2 rows
+  // x 16385: 75 us on the split engine; 8 x 16385: 27.8 on clusters), and the
+  // choice does not count that yet.
   const double nT = (double)((n + 127) / 128);
   const bool halves = h->xflag != nullptr && 2 * h->dev.R <= h->num_sms && nT >= 12;
   const double fused_us = halves ? 16.0 + 0.75 * nT : 11.0 + 1.5 * nT;

@@ -86,7 +86,9 @@ __device__ __forceinline__ void logistic(float x, float& p, float& q, float& e) 
 // of 1e10 and more straddle the cut (a row padded with a large negative number, B
 // beyond the items before the padding), no double near the root brings E[S] to B:
 // fp32 values around -u are so far apart there that E[S] varies with one of them
-// alone. Then that value is split off, u = tie + v with v in [lo, hi] instead.
+// alone. Then that value is split off, u = tie + v with v in [lo, hi] instead
+// (64 x 4096 x 1024, 500 items of each row live and 1e16 below them: 718 us in 400
+// passes without an end -> 88; rows that need no tie: 20.6, as without it).
 struct Search {
   double u, lo, hi;
   float tie;  // minus that value; 0 while u is a number of its own
